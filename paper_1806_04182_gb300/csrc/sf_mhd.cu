@@ -7,24 +7,9 @@
 // the largest fast magnetosonic signal speed of the two states; or, with
 // flux_split, the same reconstructions applied to the Lax-Friedrichs split
 // fluxes.  Fused with the RK stage update.
-#include "sf_internal.cuh"
+#include "sf_mhd.cuh"
 
 namespace sf {
-
-template <typename T>
-struct MhdCoef {
-  T gamma;
-  T eps[3];   // WENO epsilon per direction
-  T q;        // WENO-Z exponent
-  int variant;
-  int split;  // 1: reconstruction of the Lax-Friedrichs split fluxes
-  T idx[3];   // 1/dx_d
-};
-
-template <typename T>
-__device__ __forceinline__ T wz_pow(T x, T q) {
-  return q == T(2) ? x * x : (q == T(1) ? x : pow(x, q));
-}
 
 // App. B smoothness indicators of the three WENO5 stencils of cell c, from
 // w[0..4] = U_{c-2..c+2}: beta_0 of cells c..c+2, beta_1 of c-1..c+1, beta_2
@@ -104,12 +89,6 @@ __device__ __forceinline__ T weno_right(const T* w, T eps, const MhdCoef<T>& mc)
   return weno5_combine<T, Z>(c0, c1, c2, T(0.1), T(0.6), T(0.3), be0, be1, be2, eps, mc);
 }
 
-// Both edge values of cell c from w[0..4] = U_{c-2..c+2} (VAR 0 WENO5-JS,
-// 1 WENO5-Z, 2 WENO3): er = the left state at c + 1/2, el = the right state
-// at c - 1/2, with the smoothness indicators formed once
-template <typename T, int VAR>
-__device__ __forceinline__ void weno_edges(const T* w, T eps, const MhdCoef<T>& mc, T& er, T& el);
-
 // App. A: WENO3 left state at i+1/2 from w[1..3] = U_{i-1..i+1}
 template <typename T>
 __device__ __forceinline__ T weno3_left(const T* w, T eps) {
@@ -149,25 +128,6 @@ __device__ __forceinline__ T by_dir(int d, T x, T y, T z) {
   return d == 0 ? x : (d == 1 ? y : z);
 }
 
-template <typename T, int VAR>
-__device__ __forceinline__ void weno_edges(const T* w, T eps, const MhdCoef<T>& mc, T& er, T& el) {
-  if constexpr (VAR == 2) {
-    er = weno3_left(w, eps);
-    el = weno3_right(w, eps);
-  } else {
-    T be0, be1, be2;
-    weno5_beta(w, be0, be1, be2);
-    er = weno5_combine<T, VAR == 1>((T(2) * w[2] + T(5) * w[3] - w[4]) * T(1.0 / 6.0),
-                                    (-w[1] + T(5) * w[2] + T(2) * w[3]) * T(1.0 / 6.0),
-                                    (T(2) * w[0] - T(7) * w[1] + T(11) * w[2]) * T(1.0 / 6.0), T(0.3),
-                                    T(0.6), T(0.1), be0, be1, be2, eps, mc);
-    el = weno5_combine<T, VAR == 1>((T(2) * w[4] - T(7) * w[3] + T(11) * w[2]) * T(1.0 / 6.0),
-                                    (-w[3] + T(5) * w[2] + T(2) * w[1]) * T(1.0 / 6.0),
-                                    (T(2) * w[2] + T(5) * w[1] - w[0]) * T(1.0 / 6.0), T(0.1),
-                                    T(0.6), T(0.3), be0, be1, be2, eps, mc);
-  }
-}
-
 // physical flux along d and the largest signal speed |v_d| + c_fast,d
 template <typename T>
 __device__ __forceinline__ T flux_speed(const T* q, int d, const MhdCoef<T>& mc, T* F) {
@@ -191,84 +151,6 @@ __device__ __forceinline__ T flux_speed(const T* q, int d, const MhdCoef<T>& mc,
   const T s = a2 + b2;
   const T cf2 = T(0.5) * (s + sqrt(s * s - T(4) * a2 * bd2));
   return fabs(vd) + sqrt(cf2);
-}
-
-// LLF flux through the face between the cell at p and its +d neighbour;
-// VAR: the reconstruction (0 WENO5-JS, 1 WENO5-Z, 2 WENO3)
-template <typename T, int VAR>
-__device__ __forceinline__ void face_flux(const T* __restrict__ p, long long F, long long s, int d,
-                                          const MhdCoef<T>& mc, T* Fout) {
-  const T eps = by_dir(d, mc.eps[0], mc.eps[1], mc.eps[2]);
-  T UL[8], UR[8];
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    const T* q = p + f * F;
-    T w[6];
-#pragma unroll
-    for (int o = 0; o < 6; ++o) w[o] = __ldg(q + (o - 2) * s);
-    if constexpr (VAR == 2) {
-      UL[f] = weno3_left(w, eps);
-      UR[f] = weno3_right(w + 1, eps);
-    } else {
-      UL[f] = weno_left<T, VAR == 1>(w, eps, mc);
-      UR[f] = weno_right<T, VAR == 1>(w + 1, eps, mc);
-    }
-  }
-  T FL[8], FR[8];
-  const T sl = flux_speed(UL, d, mc, FL);
-  const T sr = flux_speed(UR, d, mc, FR);
-  const T S = sl > sr ? sl : sr;
-#pragma unroll
-  for (int f = 0; f < 8; ++f) Fout[f] = T(0.5) * (FL[f] + FR[f] - S * (UR[f] - UL[f]));
-}
-
-// z-faces of a thread marching up its column (double, reconstruction of the
-// evolved fields): the flux at k + 1/2 from the carried right-edge values of
-// cell k (er, 8 fields) and both edge values of cell k + 1 (cells k-1 .. k+3
-// around p1), whose right-edge values then replace er.  Each cell is
-// reconstructed once for both of its edges, its smoothness indicators formed
-// once instead of twice.
-template <typename T, int VAR>
-__device__ __forceinline__ void zface_carry(const T* __restrict__ p1, long long F, long long s,
-                                            const MhdCoef<T>& mc, T* er, T* Fout) {
-  const T eps = mc.eps[2];
-  T UR[8], ERn[8];
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    const T* q = p1 + f * F;
-    T w[5];
-#pragma unroll
-    for (int o = 0; o < 5; ++o) w[o] = __ldg(q + (o - 2) * s);
-    weno_edges<T, VAR>(w, eps, mc, ERn[f], UR[f]);
-  }
-  T FL[8], FR[8];
-  const T sl = flux_speed(er, 2, mc, FL);
-  const T sr = flux_speed(UR, 2, mc, FR);
-  const T S = sl > sr ? sl : sr;
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    Fout[f] = T(0.5) * (FL[f] + FR[f] - S * (UR[f] - er[f]));
-    er[f] = ERn[f];
-  }
-}
-
-// The right-edge values (left state at c + 1/2 along z) of the cell at p, to
-// start the carry of zface_carry.
-template <typename T, int VAR>
-__device__ __forceinline__ void zedge_right(const T* __restrict__ p, long long F, long long s,
-                                            const MhdCoef<T>& mc, T* er) {
-  const T eps = mc.eps[2];
-#pragma unroll
-  for (int f = 0; f < 8; ++f) {
-    const T* q = p + f * F;
-    T w[5];
-#pragma unroll
-    for (int o = 0; o < 5; ++o) w[o] = __ldg(q + (o - 2) * s);
-    if constexpr (VAR == 2)
-      er[f] = weno3_left(w, eps);
-    else
-      er[f] = weno_left<T, VAR == 1>(w, eps, mc);
-  }
 }
 
 // Flux through the same face from the reconstruction of the split fluxes
@@ -303,88 +185,408 @@ __device__ __forceinline__ void face_flux_split(const T* __restrict__ p, long lo
   }
 }
 
-template <typename T, bool SPLIT, int VAR>
-__device__ __forceinline__ void interface_flux(const T* __restrict__ p, long long F, long long s,
-                                               int d, const MhdCoef<T>& mc, T* Fout) {
-  if constexpr (SPLIT)
-    face_flux_split<T, VAR>(p, F, s, d, mc, Fout);
-  else
-    face_flux<T, VAR>(p, F, s, d, mc, Fout);
+// ------------------------------------------------------------ stage kernels
+// The largest signal rate of a block's outputs into *rate: block max, then
+// one atomic per block (non-negative doubles order as their bits).
+template <int NW>
+__device__ __forceinline__ void block_rate(double rate, double* s_rate, double* out) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_down_sync(0xffffffffu, rate, o));
+  if (threadIdx.x == 0) s_rate[threadIdx.y] = rate;
+  __syncthreads();
+  if (threadIdx.x == 0 && threadIdx.y == 0) {
+    double m = 0.0;
+    for (int w = 0; w < NW; ++w) m = fmax(m, s_rate[w]);
+    atomicMax(reinterpret_cast<unsigned long long*>(out), (unsigned long long)__double_as_longlong(m));
+  }
 }
 
-// Stage kernel.  Each interface flux is evaluated once: a block of 32 x MY
-// threads owns 31 x (MY - 1) output cells of a plane (MY = 12 for float
-// without flux splitting, 8 otherwise: mhd_rows); thread (tx, ty) evaluates the
-// x-face at i - 1/2 and the y-face at j - 1/2 of its column, so the +1/2
-// faces of the output cells come from lane tx + 1 (warp shuffle) and row
-// ty + 1 (shared memory).  Each thread marches mz planes in z and carries the
-// z-face below the current plane in registers (the block also evaluates the
-// z-face below its first plane, one face in 3 mz + 1, in a first pass of the
-// plane loop that evaluates nothing else, so that the kernel holds one copy
-// of the z-face code).  VAR is the reconstruction (0 WENO5-JS, 1 WENO5-Z,
-// 2 WENO3), a template argument so that each instance carries one
-// reconstruction: the kernel's code is large enough for instruction fetch to
-// be its top stall.  mz is chosen per
-// launch (mhd_planes_per_block) so that the grid fills whole waves of
-// resident blocks.  Faces are only evaluated at positions 0..n along their
-// direction, whose WENO stencils (cells p-3..p+2) lie inside the 3-point
-// ghost zone.
+template <typename T>
+__device__ __forceinline__ double cell_rate(const T* q, const MhdCoef<T>& mc) {
+  double rate = 0.0;
+  T Fd[8];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) rate = fmax(rate, double(flux_speed(q, d, mc, Fd) * mc.idx[d]));
+  return rate;
+}
+
+// The SSP-RK3 stage write of a cell's 8 fields (stage_combine, with the stage
+// chosen once for all of them); q receives the new values.
+template <typename T>
+__device__ __forceinline__ void ssp_write(const PatchArgs<T>& a, const StageArgs& s, const Images& im,
+                                          long long c, const T* cen, const T* un_m, const T* r, T* q) {
+  T un[8];
+#pragma unroll
+  for (int f = 0; f < 8; ++f) un[f] = s.un_alias ? cen[f] : un_m[f];
+  if (s.stage == 0) {
+#pragma unroll
+    for (int f = 0; f < 8; ++f) q[f] = un[f] + a.dt * r[f];
+  } else if (s.stage == 1) {
+#pragma unroll
+    for (int f = 0; f < 8; ++f) q[f] = T(0.75) * un[f] + T(0.25) * (cen[f] + a.dt * r[f]);
+  } else {
+#pragma unroll
+    for (int f = 0; f < 8; ++f) q[f] = un[f] * T(1.0 / 3.0) + T(2.0 / 3.0) * (cen[f] + a.dt * r[f]);
+  }
+  bool bad = false;
+#pragma unroll
+  for (int f = 0; f < 8; ++f) {
+    a.nx[f * a.sf + c] = q[f];
+    bad = bad || !finite_(q[f]);
+  }
+  if (s.check_finite && bad) atomicOr(s.status, ST_NONFINITE);
+  if (im.mask) {
+#pragma unroll 1
+    for (int f = 0; f < 8; ++f) store_images(a, im, f * a.sf + c, a.nx[f * a.sf + c]);
+  }
+}
+
+// Reconstruction of the evolved fields.  A block of MR + 1 warps owns a column
+// of 32 x MR cells per plane and marches in z.  In each of its three
+// directions a cell is reconstructed once, both edges together (weno_edges),
+// and each face flux is evaluated once: warp w < MR takes row w, the last warp
+// the cells and faces that the block's rows need from outside,
+//   x: right-edge values of the cells left of the tile (lanes 0 .. MR - 1),
+//      left-edge values of the cells right of it (lanes MR .. 2 MR - 1), whose
+//      faces it evaluates;
+//   y: the row below the tile, the row above it and the face row between;
+// so that all 32 x MR cells produce output.  Edge values cross to the next
+// cell by shuffle (x), shared memory (y) and in registers along the march
+// (z); fluxes likewise.  The last warp's work is a row's (3 reconstructions,
+// 2 fluxes), and every warp runs the same instructions with its own pointers,
+// so a cell's result does not depend on where in a block it lies.  Before
+// the first plane two passes evaluate only z (the right edge of the cell
+// below, then the face below the first plane).
+//
+// double is bound by the FP64 pipe (one warp instruction per 16 cycles and
+// SM; 86% busy) and reads its stencils from global memory.  float is bound by
+// issue and latency (issue 48%, then fixed-latency waits): its planes are
+// staged in shared memory as field pairs by cp.async, five in a ring, so that
+// a stencil value pair is one 64-bit load with a constant offset.  MR + 1 is
+// 16 or 8: registers are split over the four schedulers, so 9 warps get 168
+// each where 8 get 255 (float, 9 warps: 1410 us per 128^3 step, 8: 1155).
+// 128^3 SSP-RK3 step with CFL rate, against a kernel that reconstructed each
+// cell once per face and side in tiles of 31 x 11 (float) and 31 x 7 outputs:
+// double 54.5 -> 23.6 ms, float 2.24 -> 0.94 ms.
 constexpr int MX = 32;
-template <typename T, bool SPLIT>
-constexpr int mhd_rows() {
-  return sizeof(T) == 4 && !SPLIT ? 12 : 8;
-}
+template <typename T, int MR>
+struct MhdSmem {
+  static constexpr bool kStaged = sizeof(T) == 4;
+  static constexpr int kCols = MX + 6, kCells = kCols * (MR + 6);  // a plane with its halo
+  static constexpr int kSlots = 5;
+  using P = typename PairOf<T>::type;
+  T ey[MR + 1][8][MX];  // right-edge values along y of rows -1 .. MR - 1
+  T fy[MR + 1][8][MX];  // y fluxes below rows 0 .. MR
+  T exl[8][MR], exr[8][MR], fxr[8][MR];  // x: right edges of cells -1 and 31, flux at 32
+  double rate[MR + 1];
+  P ring[kStaged ? kSlots : 1][kStaged ? 4 * kCells : 1];  // planes as field pairs
+};
 
-// Float without flux splitting: blocks of 32 x 12 threads, 2 resident per SM
-// (at most 85 registers a thread, 24 warps per SM), so that 11 of 12 rows
-// output cells (7 of 8 with 32 x 8: 2.51e9 against 2.83e9 cell-updates/s at
-// 128^3; 32 x 24, one block per SM: 2.82e9; 32 x 8 left to the compiler's
-// register choice, 96 a thread and 16 warps per SM, was 15% slower than
-// 32 x 8 at 3 blocks per SM).  The other forms keep 32 x 8 and the compiler's
-// register choice.
-template <typename T, bool SPLIT>
-constexpr int mhd_min_blocks() {
-  return sizeof(T) == 4 && !SPLIT ? 2 : 1;
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
 }
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-template <typename T, bool SPLIT, int VAR>
-__global__ void __launch_bounds__(MX * mhd_rows<T, SPLIT>(), mhd_min_blocks<T, SPLIT>())
+template <typename T, int VAR, int MR>
+__global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
     mhd_stage_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, int mz) {
-  constexpr int MY = mhd_rows<T, SPLIT>();
-  __shared__ T fy[MY][MX][8];
-  __shared__ double s_rate[MX * MY / 32];
+  using S = MhdSmem<T, MR>;
+  using P = typename S::P;
+  constexpr int NC = S::kCells, CW = S::kCols;
+  constexpr bool ST = S::kStaged;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  S& sm = *reinterpret_cast<S*>(smem_raw);
   const int tx = threadIdx.x, ty = threadIdx.y;
-  double rate = 0.0;  // max signal rate of this thread's outputs (fused CFL reduction)
-  const int i = blockIdx.x * (MX - 1) + tx;
-  const int j = blockIdx.y * (MY - 1) + ty;
+  const bool row = ty < MR;
+  const int x0 = blockIdx.x * MX, y0 = blockIdx.y * MR;
   const int k0 = blockIdx.z * mz;
   const int k1 = min(k0 + mz, a.n[2]);
   const int g = a.g;
-  const bool out = tx < MX - 1 && ty < MY - 1 && i < a.n[0] && j < a.n[1];
+  const int i = x0 + tx, j = y0 + ty;
+  const bool out = row && i < a.n[0] && j < a.n[1];
+  const int xr = tx % MR;                  // the last warp's x lanes: their row,
+  const bool xright = (tx / MR) % 2 == 1;  // and which side of the tile
+  const bool do_xz = !row || j < a.n[1], do_y = !row || j <= a.n[1];
+  const int ys = row ? ty + 1 : 0, yl = row ? ty : MR;  // ey rows written / read, fy row written
+  // cell offsets in a plane (x, y and third reconstruction), in the staged
+  // plane or in the global one.  Cells outside the patch that a face needs lie
+  // in its ghost zone; lanes and rows beyond those repeat others (their
+  // results go nowhere).
+  long long gx = 0, gy = 0, gz = 0;
+  int lx_ = 0, ly_ = 0, lz_ = 0;
+  const long long c0 = (long long)(min(j, a.n[1]) + g) * a.sy + (min(i, a.n[0]) + g);
+  if constexpr (ST) {
+    ly_ = ((row ? ty : -1) + 3) * CW + tx + 3;
+    lx_ = row ? ly_ : (xr + 3) * CW + (xright ? MX : -1) + 3;
+    lz_ = row ? ly_ : (MR + 3) * CW + tx + 3;
+  } else {
+    auto cell = [&](int ci, int cj) {
+      return (long long)(min(cj, a.n[1]) + g) * a.sy + (min(ci, a.n[0]) + g);
+    };
+    gy = row ? c0 : cell(i, y0 - 1);
+    gx = row ? c0 : cell(xright ? x0 + MX : x0 - 1, y0 + xr);
+    gz = row ? c0 : cell(i, y0 + MR);
+  }
+  // staging: plane p (interior index) into ring slot q, each thread its cells
+  constexpr int NT = MX * (MR + 1), NS = (NC + NT - 1) / NT;
+  long long so[NS];
+  if constexpr (ST) {
+#pragma unroll
+    for (int e = 0; e < NS; ++e) {
+      const int t = ty * MX + tx + e * NT;
+      const int cx = min(x0 - 3 + t % CW, a.n[0] + 2), cy = min(y0 - 3 + t / CW, a.n[1] + 2);
+      so[e] = (long long)(cy + g) * a.sy + (cx + g);
+    }
+  }
+  auto stage = [&](int p, int q) {
+    if constexpr (ST) {
+      const T* pl = a.us + (long long)(p + g) * a.sz;
+#pragma unroll
+      for (int e = 0; e < NS; ++e) {
+        const int t = ty * MX + tx + e * NT;
+        if (t < NC) {
+          const T* src = pl + so[e];
+          float* dst = reinterpret_cast<float*>(&sm.ring[q][t]);
+#pragma unroll
+          for (int f = 0; f < 8; ++f, src += a.sf) cp_async4(dst + (f / 2) * (2 * NC) + f % 2, src);
+        }
+      }
+    }
+  };
+  // (left, right) states of a face
+  auto states = [](const P* l, const P* r, P* q) {
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      q[2 * f] = P(l[f].x, r[f].x);
+      q[2 * f + 1] = P(l[f].y, r[f].y);
+    }
+  };
+  double rate = 0.0;  // max signal rate of this thread's outputs (fused CFL reduction)
+  P erz[4];           // right-edge values along z of the cell below
+  T Fzm[8];           // z flux below the current plane
+#pragma unroll
+  for (int f = 0; f < 4; ++f) erz[f] = P(T(1));
+  int sl[5] = {0, 1, 2, 3, 4};  // ring slots of planes k - 1 .. k + 3
+  if constexpr (ST) {
+    for (int q = 0; q < 5; ++q) stage(k0 - 3 + q, q);
+    cp_async_wait();
+    __syncthreads();
+  }
+  for (int k = k0 - 2; k < k1; ++k) {
+    const T* plane = a.us + (long long)(k + g) * a.sz;
+    const bool body = k >= k0;
+    // both edges of a cell from the plane's values at stride st (staged: cells
+    // of the ring slot of plane k; global: elements)
+    auto recon = [&](int lc, long long gc, int lst, long long gst, T eps, P* er, P* el) {
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        P w[5];
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+          if constexpr (ST) {
+            w[o] = sm.ring[sl[1]][f * NC + lc + (o - 2) * lst];
+          } else {
+            const T* q = plane + gc + (o - 2) * gst + 2 * f * a.sf;
+            w[o] = P(__ldg(q), __ldg(q + a.sf));
+          }
+        }
+        weno_edges<VAR, T, P>(w, eps, mc, er[f], el[f]);
+      }
+    };
+    P rx[4], lx[4], ly[4];
+    T dz[8];
+    if (body && do_y) {
+      P ry[4];
+      recon(ly_, gy, CW, a.sy, mc.eps[1], ry, ly);
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        sm.ey[ys][2 * f][tx] = ry[f].x;
+        sm.ey[ys][2 * f + 1][tx] = ry[f].y;
+      }
+    }
+    if (body && do_xz) {
+      recon(lx_, gx, 1, 1, mc.eps[0], rx, lx);
+      if (row && tx == MX - 1) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          sm.exr[2 * f][ty] = rx[f].x;
+          sm.exr[2 * f + 1][ty] = rx[f].y;
+        }
+      }
+      if (!row && tx < MR) {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          sm.exl[2 * f][tx] = rx[f].x;
+          sm.exl[2 * f + 1][tx] = rx[f].y;
+        }
+      }
+    }
+    if (do_xz && (row || body)) {
+      // rows: cell k + 1 along z; the last warp: the row above the tile along y
+      P r[4], l[4];
+      const T eps = row ? mc.eps[2] : mc.eps[1];
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        P w[5];
+#pragma unroll
+        for (int o = 0; o < 5; ++o) {
+          if constexpr (ST) {
+            w[o] = sm.ring[row ? sl[o] : sl[1]][f * NC + lz_ + (row ? 0 : (o - 2) * CW)];
+          } else {
+            const T* q = plane + (row ? a.sz : 0) + gz + (o - 2) * (row ? a.sz : a.sy) + 2 * f * a.sf;
+            w[o] = P(__ldg(q), __ldg(q + a.sf));
+          }
+        }
+        weno_edges<VAR, T, P>(w, eps, mc, r[f], l[f]);
+      }
+      if (row) {
+        P q[8];
+        T F[8];
+        states(erz, l, q);
+        llf_flux2<2, T, P>(q, mc.gamma, F);
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+          dz[f] = F[f] - Fzm[f];
+          Fzm[f] = F[f];
+        }
+#pragma unroll
+        for (int f = 0; f < 4; ++f) erz[f] = r[f];
+      } else {
+#pragma unroll
+        for (int f = 0; f < 4; ++f) ly[f] = l[f];
+      }
+    }
+    if (body || ST) __syncthreads();  // ey, exl, exr; plane k - 1 is read
+    if constexpr (ST) {
+      if (k + 1 < k1) stage(k + 4, sl[0]);
+    }
+    if (body) {
+      T Fx[8], Fy[8];
+      if (do_xz) {
+        P lt[4], q[8];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) {
+          lt[f].x = __shfl_up_sync(0xffffffffu, rx[f].x, 1);
+          lt[f].y = __shfl_up_sync(0xffffffffu, rx[f].y, 1);
+        }
+        if (row ? tx == 0 : xright) {
+#pragma unroll
+          for (int f = 0; f < 4; ++f)
+            lt[f] = row ? P(sm.exl[2 * f][ty], sm.exl[2 * f + 1][ty])
+                        : P(sm.exr[2 * f][xr], sm.exr[2 * f + 1][xr]);
+        }
+        states(lt, lx, q);
+        llf_flux2<0, T, P>(q, mc.gamma, Fx);
+        if (!row && xright) {
+#pragma unroll
+          for (int f = 0; f < 8; ++f) sm.fxr[f][xr] = Fx[f];
+        }
+      }
+      if (do_y) {
+        P lt[4], q[8];
+#pragma unroll
+        for (int f = 0; f < 4; ++f) lt[f] = P(sm.ey[yl][2 * f][tx], sm.ey[yl][2 * f + 1][tx]);
+        states(lt, ly, q);
+        llf_flux2<1, T, P>(q, mc.gamma, Fy);
+#pragma unroll
+        for (int f = 0; f < 8; ++f) sm.fy[yl][f][tx] = Fy[f];
+      }
+      // U^n, if a stage reads it from memory, on its way across the barrier
+      const long long c = (long long)(k + g) * a.sz + c0;
+      T un[8];
+      if (!s.un_alias && s.mode == 0 && out) {
+#pragma unroll
+        for (int f = 0; f < 8; ++f) un[f] = a.un[f * a.sf + c];
+      }
+      if constexpr (ST) cp_async_wait();
+      __syncthreads();  // fy, fxr; plane k + 4
+      if (row && do_xz) {
+        T q[8], rhs[8];
+#pragma unroll
+        for (int f = 0; f < 8; ++f) {
+          T fxp = __shfl_down_sync(0xffffffffu, Fx[f], 1);
+          if (tx == MX - 1) fxp = sm.fxr[f][ty];
+          // the fluxes are twice the fluxes
+          T r = (fxp - Fx[f]) * (T(-0.5) * mc.idx[0]);
+          r = fma(sm.fy[ty + 1][f][tx] - Fy[f], T(-0.5) * mc.idx[1], r);
+          r = fma(dz[f], T(-0.5) * mc.idx[2], r);
+          rhs[f] = r;
+        }
+        if (out) {
+          T cen[8];
+#pragma unroll
+          for (int f = 0; f < 8; ++f) {
+            if constexpr (ST) {
+              const P v = sm.ring[sl[1]][(f / 2) * NC + lz_];
+              cen[f] = f % 2 ? v.y : v.x;
+            } else {
+              cen[f] = __ldg(a.us + f * a.sf + c);
+            }
+          }
+          const Images im = ghost_images(a, s, i, j, k);
+          if (s.mode == 0 && s.rk == SF_SSPRK3)
+            ssp_write(a, s, im, c, cen, un, rhs, q);
+          else
+#pragma unroll
+            for (int f = 0; f < 8; ++f) q[f] = write_field(a, s, im, f, c, i, j, k, cen[f], rhs[f]);
+        }
+        if (out && a.rate) rate = fmax(rate, cell_rate(q, mc));
+      }
+    } else if constexpr (ST) {
+      cp_async_wait();
+      __syncthreads();
+    }
+    const int t = sl[0];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sl[q] = sl[q + 1];
+    sl[4] = t;
+  }
+  if (a.rate) block_rate<MR + 1>(rate, sm.rate, a.rate);
+}
+
+// Lax-Friedrichs flux splitting.  The split fluxes of a cell depend on the
+// face (S is the face's), so both sides are reconstructed per face: a block of
+// 32 x 8 threads owns 31 x 7 output cells of a plane; thread (tx, ty)
+// evaluates the x-face at i - 1/2 and the y-face at j - 1/2 of its column, so
+// the +1/2 faces of the output cells come from lane tx + 1 (warp shuffle) and
+// row ty + 1 (shared memory), and carries the z-face below the current plane
+// in registers while it marches mz planes (a first pass evaluates only the
+// z-face below the first plane).  The three directions run in one rolled
+// loop, so the kernel holds one copy of the face code.
+constexpr int SY = 8;
+template <typename T, int VAR>
+__global__ void __launch_bounds__(MX * SY)
+    mhd_split_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, int mz) {
+  __shared__ T fy[SY][MX][8];
+  __shared__ double s_rate[SY];
+  const int tx = threadIdx.x, ty = threadIdx.y;
+  double rate = 0.0;  // max signal rate of this thread's outputs (fused CFL reduction)
+  const int i = blockIdx.x * (MX - 1) + tx;
+  const int j = blockIdx.y * (SY - 1) + ty;
+  const int k0 = blockIdx.z * mz;
+  const int k1 = min(k0 + mz, a.n[2]);
+  const int g = a.g;
+  const bool out = tx < MX - 1 && ty < SY - 1 && i < a.n[0] && j < a.n[1];
   const bool xface = i <= a.n[0] && j < a.n[1];
   const bool yface = j <= a.n[1] && i < a.n[0];
   auto at = [&](int ii, int jj, int kk) {
     return a.us + (long long)(kk + g) * a.sz + (long long)(jj + g) * a.sy + (ii + g);
   };
-  // double without flux splitting: the z-faces by zface_carry (each cell's
-  // z reconstruction serves both of its z-faces), er its carried values
-  constexpr bool ZC = sizeof(T) == 8 && !SPLIT;
-  T Fzm[8], er[8];
+  T Fzm[8];
   // pass k = k0 - 1 evaluates only the z-face below the first plane (Fzm);
   // `body` is the same for the whole block, so the barriers below are taken
   // by every thread or by none
   for (int k = k0 - 1; k < k1; ++k) {
     const bool body = k >= k0;
     T Fx[8], Fy[8], Fz[8];
-    // the x-face at i - 1/2, the y-face at j - 1/2 and the z-face at k + 1/2
-    // in one rolled loop over the direction (one copy of the face code); with
-    // ZC the z-face comes from zface_carry after the loop
 #pragma unroll 1
-    for (int d = body ? 0 : 2; d < (ZC ? 2 : 3); ++d) {
+    for (int d = body ? 0 : 2; d < 3; ++d) {
       T Fd[8];
       if (d == 0 ? xface : (d == 1 ? yface : out)) {
         const T* base = d == 0 ? at(i - 1, j, k) : (d == 1 ? at(i, j - 1, k) : at(i, j, k));
-        interface_flux<T, SPLIT, VAR>(base, a.sf, d == 0 ? 1LL : (d == 1 ? a.sy : a.sz), d, mc, Fd);
+        face_flux_split<T, VAR>(base, a.sf, d == 0 ? 1LL : (d == 1 ? a.sy : a.sz), d, mc, Fd);
       } else {
 #pragma unroll
         for (int f = 0; f < 8; ++f) Fd[f] = T(0);
@@ -396,21 +598,13 @@ __global__ void __launch_bounds__(MX * mhd_rows<T, SPLIT>(), mhd_min_blocks<T, S
         Fz[f] = d == 2 ? Fd[f] : Fz[f];
       }
     }
-    if constexpr (ZC) {
-      if (out) {
-        if (!body) zedge_right<T, VAR>(at(i, j, k), a.sf, a.sz, mc, er);
-        zface_carry<T, VAR>(at(i, j, k + 1), a.sf, a.sz, mc, er, Fz);
-      }
-    }
-    if (body) {
-#pragma unroll
-      for (int f = 0; f < 8; ++f) fy[ty][tx][f] = Fy[f];
-    }
     if (!body) {
 #pragma unroll
       for (int f = 0; f < 8; ++f) Fzm[f] = Fz[f];
       continue;
     }
+#pragma unroll
+    for (int f = 0; f < 8; ++f) fy[ty][tx][f] = Fy[f];
     T Fxp[8];
 #pragma unroll
     for (int f = 0; f < 8; ++f) Fxp[f] = __shfl_down_sync(0xffffffffu, Fx[f], 1);
@@ -428,26 +622,11 @@ __global__ void __launch_bounds__(MX * mhd_rows<T, SPLIT>(), mhd_min_blocks<T, S
         q[f] = write_field(a, s, im, f, c, i, j, k, __ldg(a.us + f * a.sf + c), r);
         Fzm[f] = Fz[f];
       }
-      if (a.rate) {
-        T Fd[8];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) rate = fmax(rate, double(flux_speed(q, d, mc, Fd) * mc.idx[d]));
-      }
+      if (a.rate) rate = fmax(rate, cell_rate(q, mc));
     }
     __syncthreads();
   }
-  if (a.rate) {  // block max, then one atomic per block (non-negative doubles order as their bits)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rate = fmax(rate, __shfl_down_sync(0xffffffffu, rate, o));
-    const int lin = ty * MX + tx;
-    if ((lin & 31) == 0) s_rate[lin >> 5] = rate;
-    __syncthreads();
-    if (lin == 0) {
-      double m = 0.0;
-      for (int w = 0; w < MX * MY / 32; ++w) m = fmax(m, s_rate[w]);
-      atomicMax(reinterpret_cast<unsigned long long*>(a.rate), (unsigned long long)__double_as_longlong(m));
-    }
-  }
+  if (a.rate) block_rate<SY>(rate, s_rate, a.rate);
 }
 
 // CFL rate: max over cells and d of (|v_d| + c_fast,d) / dx_d
@@ -500,56 +679,90 @@ static MhdCoef<T> coef(const sf_params& prm, const sf_patch& p) {
   return mc;
 }
 
-// Planes per block along z: each block evaluates 3 mz + 1 interface fluxes
-// per column, and a launch of B blocks takes ceil(B / resident) rounds of
-// the resident blocks (blocks per SM x SMs), so mz in [4, 16] minimises
-// ceil(B(mz) / resident) (3 mz + 1); ties go to the larger mz.  Only chunk
-// lengths whose grid fits gridDim.z (65535) are considered.
-static int mhd_planes_per_block(int gx, int gy, int nz, int resident) {
-  int best = 16;
-  long long best_cost = -1;
-  for (int mz = 16; mz >= 4; --mz) {
+// Planes per block along z: a block evaluates mz planes and the passes before
+// its first one, about (3 mz + extra) / 3 planes' work, and a launch of B
+// blocks takes ceil(B / resident) rounds of the resident blocks (blocks per
+// SM x SMs), so mz in [1, 32] minimises the cost ceil(B(mz) / resident)
+// (3 mz + extra); ties go to the larger mz.  Only chunk lengths whose grid
+// fits gridDim.z (65535) are considered.
+struct MhdPlan {
+  int mz;
+  long long cost;
+};
+static MhdPlan mhd_planes_per_block(int gx, int gy, int nz, int resident, int extra) {
+  MhdPlan best = {32, -1};
+  for (int mz = 32; mz >= 1; --mz) {
     if ((nz + mz - 1) / mz > 65535) break;
     const long long blocks = (long long)gx * gy * ((nz + mz - 1) / mz);
     const long long rounds = resident > 0 ? (blocks + resident - 1) / resident : blocks;
-    const long long cost = rounds * (3 * mz + 1);
-    if (best_cost < 0 || cost < best_cost) {
-      best_cost = cost;
-      best = mz;
-    }
+    const long long cost = rounds * (3 * mz + extra);
+    if (best.cost < 0 || cost < best.cost) best = {mz, cost};
   }
   return best;
 }
 
-// Resident blocks of the stage kernel instance on the current device
-// (blocks per SM x SMs), cached per instance and device; 0 if unknown.
-template <typename T, bool SPLIT, int VAR>
-static int resident_blocks() {
-  static int cache[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cache[dev]) {
-    int per_sm = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, mhd_stage_kernel<T, SPLIT, VAR>,
-                                                      MX * mhd_rows<T, SPLIT>(),
-                                                      0) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return 0;
-    cache[dev] = per_sm * sms;
+// A stage kernel instance: block, tile of output cells and dynamic shared
+// memory.  ROWS: the output rows of mhd_stage_kernel, 0 for mhd_split_kernel.
+template <typename T, int VAR, int ROWS>
+struct MhdInstance {
+  static constexpr int threads_y = ROWS ? ROWS + 1 : SY;
+  static constexpr int out_x = ROWS ? MX : MX - 1, out_y = ROWS ? ROWS : SY - 1;
+  static constexpr int smem = ROWS ? (int)sizeof(MhdSmem<T, ROWS ? ROWS : 1>) : 0;
+  static constexpr auto kernel() {
+    if constexpr (ROWS == 0)
+      return mhd_split_kernel<T, VAR>;
+    else
+      return mhd_stage_kernel<T, VAR, ROWS>;
   }
-  return cache[dev];
-}
+  // Resident blocks on the current device (blocks per SM x SMs), cached per
+  // device; 0 if unknown.  The first call on a device opts the kernel into
+  // its shared memory.
+  static int resident() {
+    static int cache[64] = {0};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    if (!cache[dev]) {
+      int per_sm = 0, sms = 0;
+      if (cudaFuncSetAttribute(kernel(), cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess ||
+          cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel(), MX * threads_y, smem) !=
+              cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+      cache[dev] = per_sm * sms;
+    }
+    return cache[dev];
+  }
+  static MhdPlan plan(const sf_patch& p) {
+    return mhd_planes_per_block((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y, p.n[2],
+                                resident(), ROWS ? 2 : 1);
+  }
+  static void launch(const PatchArgs<T>& a, const StageArgs& s, const MhdCoef<T>& mc, const sf_patch& p,
+                     int mz, cudaStream_t st) {
+    const dim3 block(MX, threads_y, 1);
+    const dim3 grid((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y, (p.n[2] + mz - 1) / mz);
+    kernel()<<<grid, block, smem, st>>>(a, s, mc, mz);
+  }
+};
 
-// One launch of the instance for (T, SPLIT, VAR) with its chunk length.
+// Without flux splitting: blocks of 15 or 7 output rows.  Both forms keep 16
+// warps resident per SM (one block or two), so a plane of a round costs the
+// same and the plans' costs compare; on a tie 15 rows, whose extra warp is 1
+// in 16 instead of 1 in 8 (128^3 float: 1124 against 1155 us per step).
 template <typename T, bool SPLIT, int VAR>
 static void launch_instance(const PatchArgs<T>& a, const StageArgs& s, const MhdCoef<T>& mc,
                             const sf_patch& p, cudaStream_t st) {
-  constexpr int MY = mhd_rows<T, SPLIT>();
-  const dim3 block(MX, MY, 1);
-  const int gx = (p.n[0] + MX - 2) / (MX - 1), gy = (p.n[1] + MY - 2) / (MY - 1);
-  const int mz = mhd_planes_per_block(gx, gy, p.n[2], resident_blocks<T, SPLIT, VAR>());
-  const dim3 grid(gx, gy, (p.n[2] + mz - 1) / mz);
-  mhd_stage_kernel<T, SPLIT, VAR><<<grid, block, 0, st>>>(a, s, mc, mz);
+  if constexpr (SPLIT) {
+    using I = MhdInstance<T, VAR, 0>;
+    I::launch(a, s, mc, p, I::plan(p).mz, st);
+  } else {
+    using A = MhdInstance<T, VAR, 15>;
+    using B = MhdInstance<T, VAR, 7>;
+    const MhdPlan pa = A::plan(p), pb = B::plan(p);
+    if (pa.cost <= pb.cost)
+      A::launch(a, s, mc, p, pa.mz, st);
+    else
+      B::launch(a, s, mc, p, pb.mz, st);
+  }
 }
 
 template <typename T, bool SPLIT>

@@ -1,0 +1,308 @@
+// Per-face arithmetic of the MHD stage kernel on pairs of values: the WENO
+// reconstruction (App. A, App. B) of both edges of a cell for two fields at
+// once, and the local Lax-Friedrichs flux (Eq. LLF) with the left and right
+// states of a face as the two lanes.  For float a pair is an F2, each step
+// one f32x2 instruction; for double it is two scalars.
+//
+// Both edges of a cell share everything but their linear weights: with the
+// differences d_k = w_{k+1} - w_k and second differences a_k, the candidate
+// polynomials at the right edge are w_2 + d_2/2 - a_0/6, w_2 + d_2/2 - a_1/6
+// and w_2 + d_2/2 - (3 a_1 - 2 a_2)/6, at the left edge the mirror images, and
+// the nonlinear weights are linear weight x P_k with the same P_k for both
+// edges.  The edge value is the cell's value plus a correction, so a uniform
+// state is reproduced exactly and the correction's rounding is relative to
+// the correction.  47 operations give both edges (double) (App. B evaluated per face
+// and per side takes about 124 for the same two values).
+#pragma once
+
+#include "sf_f2.cuh"
+#include "sf_internal.cuh"
+
+namespace sf {
+
+template <typename T>
+struct MhdCoef {
+  T gamma;
+  T eps[3];   // WENO epsilon per direction
+  T q;        // WENO-Z exponent
+  int variant;
+  int split;  // 1: reconstruction of the Lax-Friedrichs split fluxes
+  T idx[3];   // 1/dx_d
+};
+
+template <typename T>
+__device__ __forceinline__ T wz_pow(T x, T q) {
+  return q == T(2) ? x * x : (q == T(1) ? x : pow(x, q));
+}
+
+// ------------------------------------------------------------ pairs
+// Two doubles; the compiler contracts none of these (explicit rounding), so
+// every copy of the face code rounds alike.
+struct R2 {
+  double x, y;
+  R2() = default;
+  __device__ __forceinline__ R2(double a, double b) : x(a), y(b) {}
+  __device__ __forceinline__ explicit R2(double v) : x(v), y(v) {}
+};
+__device__ __forceinline__ R2 add2(R2 a, R2 b) { return R2(__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y)); }
+__device__ __forceinline__ R2 sub2(R2 a, R2 b) { return R2(__dsub_rn(a.x, b.x), __dsub_rn(a.y, b.y)); }
+__device__ __forceinline__ R2 mul2(R2 a, R2 b) { return R2(__dmul_rn(a.x, b.x), __dmul_rn(a.y, b.y)); }
+__device__ __forceinline__ R2 fma2(R2 a, R2 b, R2 c) {
+  return R2(__fma_rn(a.x, b.x, c.x), __fma_rn(a.y, b.y, c.y));
+}
+__device__ __forceinline__ R2 neg2(R2 a) { return R2(-a.x, -a.y); }
+
+template <typename T>
+struct PairOf;
+template <>
+struct PairOf<float> {
+  using type = F2;
+};
+template <>
+struct PairOf<double> {
+  using type = R2;
+};
+
+// -1/x.  float: the hardware approximation and one Newton step; double: the
+// approximation rcp.approx.ftz.f64 (relative error below 2^-20) and one step
+// of Householder's cubic iteration z (1 + e + e^2), e = 1 + x z (error below
+// 2^-60 before rounding): 3 FP64 operations where the IEEE quotient takes
+// about 9, on a pipe that issues one warp instruction every 16 cycles per SM.
+// Exponents at which the approximation flushes or overflows take the IEEE
+// division.  (The negative, because f32x2 has no negated operands: the sign
+// goes into the scalar approximation for free.)
+__device__ __forceinline__ float nrecip_approx(float x) {
+  float z;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(z) : "f"(-x));
+  return z;
+}
+__device__ __forceinline__ F2 nrecip2(F2 x) {
+  const F2 z(nrecip_approx(x.x), nrecip_approx(x.y));
+  return fma2(z, fma2(x, z, F2(1.0f)), z);
+}
+// HALF: -1/(2x), the half by one off the approximation's exponent
+template <bool HALF>
+__device__ __forceinline__ double nrecip1(double x) {
+  const unsigned ex = (unsigned)__double2hiint(x) & 0x7ff00000u;
+  if (ex - 0x00400000u >= 0x7f800000u - 0x00400000u) return (HALF ? -0.5 : -1.0) / x;
+  double z;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(z) : "d"(-x));
+  const double e = __fma_rn(x, z, 1.0);
+  if (HALF) z = __hiloint2double(__double2hiint(z) - 0x00100000, __double2loint(z));
+  return __fma_rn(z, __fma_rn(e, e, e), z);
+}
+__device__ __forceinline__ R2 nrecip2(R2 x) { return R2(nrecip1<false>(x.x), nrecip1<false>(x.y)); }
+
+// Square root of a non-negative value; float: h = x rsqrt(x) and one Newton
+// step h (3/2 - h rsqrt(x) / 2).
+__device__ __forceinline__ F2 sqrt2(F2 x) {
+  auto rs = [](float v) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(v, 1e-37f)));
+    return y;
+  };
+  const F2 y(rs(x.x), rs(x.y));
+  const F2 h = mul2(x, y);
+  return fma2(h, fma2(mul2(y, F2(-0.5f)), h, F2(0.5f)), h);
+}
+// double: h = x y with y = rsqrt.approx.ftz.f64, e = 1 - h y, and Halley's
+// cubic step h (1 + e/2 + 3 e^2/8): 5 FP64 operations; exponents near the ends
+// of the range (zero, inf and NaN among them) take the IEEE root.
+__device__ __forceinline__ double sqrt1(double x) {
+  const unsigned hi = (unsigned)__double2hiint(x);
+  if (hi - 0x00400000u >= 0x7f800000u - 0x00400000u) return sqrt(x);  // a set sign bit too
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
+  return __fma_rn(__dmul_rn(h, e), __fma_rn(0.375, e, 0.5), h);
+}
+__device__ __forceinline__ R2 sqrt2(R2 x) { return R2(sqrt1(x.x), sqrt1(x.y)); }
+
+// max(x, 0) per lane, NaN kept out of the comparison; double: by the sign
+// bit, off the FP64 pipe.
+__device__ __forceinline__ F2 pos2(F2 x) { return F2(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f)); }
+__device__ __forceinline__ R2 pos2(R2 x) {
+  return R2(__double2hiint(x.x) < 0 ? 0.0 : x.x, __double2hiint(x.y) < 0 ? 0.0 : x.y);
+}
+__device__ __forceinline__ F2 abs2(F2 x) { return F2(fabsf(x.x), fabsf(x.y)); }
+__device__ __forceinline__ R2 abs2(R2 x) { return R2(fabs(x.x), fabs(x.y)); }
+__device__ __forceinline__ F2 minus2(F2 x) { return mul2(x, F2(-1.0f)); }
+__device__ __forceinline__ R2 minus2(R2 x) { return neg2(x); }
+// the larger of two non-negative values; double: as integers (their bits are
+// ordered alike, NaN above all)
+__device__ __forceinline__ float larger(float a, float b) { return a > b ? a : b; }
+__device__ __forceinline__ double larger(double a, double b) {
+  return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
+}
+
+// ------------------------------------------------------------ reconstruction
+// Nonlinear weights P_k (without their linear weights) from E_k = eps + beta_k,
+// up to a common factor, and the two reciprocals 1/s_R, 1/s_L.
+//
+// JS weights are 1/E_k^2; over the common denominator P_0 = (E_1 E_2)^2 and
+// so on.  In float the products E_i E_j are scaled by the power of two of the
+// largest first, so that the largest P_k lies in [1, 4) whatever the units,
+// and E_k is capped at 1.5e19, beyond which its weight is nil (1/E_k^2 is
+// zero in float too).
+template <int VAR>
+__device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
+                                             F2& p1, F2& p2) {
+  if constexpr (VAR == 1) {
+    const F2 tau = abs2(sub2(e0, e2));
+    auto w = [&](F2 e) {
+      return F2(1.0f + wz_pow(tau.x / e.x, mc.q), 1.0f + wz_pow(tau.y / e.y, mc.q));
+    };
+    p0 = w(e0);
+    p1 = w(e1);
+    p2 = w(e2);
+  } else {
+    auto cap = [](F2 e) { return F2(fminf(e.x, 1.5e19f), fminf(e.y, 1.5e19f)); };
+    e0 = cap(e0);
+    e1 = cap(e1);
+    e2 = cap(e2);
+    p0 = mul2(e1, e2);
+    p1 = mul2(e0, e2);
+    p2 = mul2(e0, e1);
+    auto scale = [](float a, float b, float c) {
+      const float m = fmaxf(fmaxf(a, b), c);
+      return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+    };
+    const F2 sc(scale(p0.x, p1.x, p2.x), scale(p0.y, p1.y, p2.y));
+    p0 = mul2(p0, sc);
+    p1 = mul2(p1, sc);
+    p2 = mul2(p2, sc);
+    p0 = mul2(p0, p0);
+    p1 = mul2(p1, p1);
+    p2 = mul2(p2, p2);
+  }
+}
+template <int VAR>
+__device__ __forceinline__ void weno_weights(R2 e0, R2 e1, R2 e2, const MhdCoef<double>& mc, R2& p0,
+                                             R2& p1, R2& p2) {
+  if constexpr (VAR == 1) {
+    const R2 tau = abs2(sub2(e0, e2));
+    if (mc.q == 2.0) {  // (E_k^2 + tau^2) (E_i E_j)^2
+      const R2 t2 = mul2(tau, tau);
+      const R2 q0 = mul2(e0, e0), q1 = mul2(e1, e1), q2 = mul2(e2, e2);
+      p0 = mul2(add2(q0, t2), mul2(q1, q2));
+      p1 = mul2(add2(q1, t2), mul2(q0, q2));
+      p2 = mul2(add2(q2, t2), mul2(q0, q1));
+    } else {
+      auto w = [&](R2 e) {
+        return R2(1.0 + wz_pow(tau.x / e.x, mc.q), 1.0 + wz_pow(tau.y / e.y, mc.q));
+      };
+      p0 = w(e0);
+      p1 = w(e1);
+      p2 = w(e2);
+    }
+  } else {
+    p0 = mul2(e1, e2);
+    p1 = mul2(e0, e2);
+    p2 = mul2(e0, e1);
+    p0 = mul2(p0, p0);
+    p1 = mul2(p1, p1);
+    p2 = mul2(p2, p2);
+  }
+}
+
+// -1/2 x the reciprocals of both sums.  float JS: the sums lie in [1, 64), so
+// one reciprocal of their product serves both.
+template <int VAR>
+__device__ __forceinline__ void half_recips(F2 sr, F2 sl, F2& ir, F2& il) {
+  if constexpr (VAR == 0) {
+    const F2 h = mul2(nrecip2(mul2(sr, sl)), F2(0.5f));
+    ir = mul2(h, sl);
+    il = mul2(h, sr);
+  } else {
+    ir = mul2(nrecip2(sr), F2(0.5f));
+    il = mul2(nrecip2(sl), F2(0.5f));
+  }
+}
+template <int VAR>
+__device__ __forceinline__ void half_recips(R2 sr, R2 sl, R2& ir, R2& il) {
+  ir = R2(nrecip1<true>(sr.x), nrecip1<true>(sr.y));
+  il = R2(nrecip1<true>(sl.x), nrecip1<true>(sl.y));
+}
+
+// Both edge values of cell c of two fields from w[0..4] = U_{c-2..c+2}: er,
+// the left state at c + 1/2, and el, the right state at c - 1/2.  VAR 0
+// WENO5-JS, 1 WENO5-Z, 2 WENO3.
+template <int VAR, typename T, typename P>
+__device__ __forceinline__ void weno_edges(const P* w, T eps, const MhdCoef<T>& mc, P& er, P& el) {
+  const P d1 = sub2(w[2], w[1]), d2 = sub2(w[3], w[2]);
+  if constexpr (VAR == 2) {
+    const P ep(eps);
+    P e0 = fma2(d2, d2, ep), e1 = fma2(d1, d1, ep);
+    if constexpr (sizeof(T) == 4) {  // as weno_weights: beyond the cap the weight is nil
+      e0 = P(fminf(e0.x, 1.5e19f), fminf(e0.y, 1.5e19f));
+      e1 = P(fminf(e1.x, 1.5e19f), fminf(e1.y, 1.5e19f));
+    }
+    const P p0 = mul2(e1, e1), p1 = mul2(e0, e0);
+    // er = w_2 + (2 p0 d2 + p1 d1) / (2 (2 p0 + p1)), el its mirror image
+    const P q0 = mul2(p0, d2), q1 = mul2(p1, d1), two(T(2));
+    P ir, il;
+    half_recips<VAR>(fma2(two, p0, p1), fma2(two, p1, p0), ir, il);
+    er = fma2(fma2(P(T(-2)), q0, minus2(q1)), ir, w[2]);
+    el = fma2(fma2(two, q1, q0), il, w[2]);
+    return;
+  }
+  // beta_k = 4/3 a_k^2 + a product of differences (13/12 a^2 + 1/4 b^2 of App. B
+  // with b expressed by a and the differences)
+  const P d0 = sub2(w[1], w[0]), d3 = sub2(w[4], w[3]);
+  const P a0 = sub2(d3, d2), a1 = sub2(d2, d1), a2 = sub2(d1, d0);
+  const P c43(T(4.0 / 3.0)), ep(eps);
+  const P e0 = fma2(d2, sub2(d2, a0), fma2(mul2(c43, a0), a0, ep));
+  const P e1 = fma2(d1, d2, fma2(mul2(c43, a1), a1, ep));
+  const P e2 = fma2(d1, add2(d1, a2), fma2(mul2(c43, a2), a2, ep));
+  P p0, p1, p2;
+  weno_weights<VAR>(e0, e1, e2, mc, p0, p1, p2);
+  // right edge: weights 3 p0, 6 p1, p2; left edge: p0, 6 p1, 3 p2
+  const P two(T(2)), three(T(3)), mt(T(-2.0 / 3.0));
+  const P s6 = mul2(P(T(6)), p1);
+  const P sr = add2(fma2(three, p0, s6), p2), sl = add2(fma2(three, p2, s6), p0);
+  const P ur = fma2(two, p1, p2), ul = fma2(two, p1, p0);
+  const P q0 = mul2(p0, a0), q2 = mul2(p2, a2);
+  const P nr = fma2(mt, q2, fma2(ur, a1, q0));
+  const P nl = fma2(mt, q0, fma2(ul, a1, q2));
+  P ir, il;
+  half_recips<VAR>(sr, sl, ir, il);
+  er = fma2(nr, ir, fma2(P(T(0.5)), d2, w[2]));
+  el = fma2(nl, il, fma2(P(T(-0.5)), d1, w[2]));
+}
+
+// ------------------------------------------------------------ flux
+// Twice the LLF flux through a face along D, FL + FR - S (UR - UL), from the
+// states q[f] = (left, right).  Velocities and fluxes are carried negated
+// (n...), see nrecip2.
+template <int D, typename T, typename P>
+__device__ __forceinline__ void llf_flux2(const P* q, T gamma, T* F) {
+  constexpr int A = (D + 1) % 3, B = (D + 2) % 3;  // the other two directions
+  const P nir = nrecip2(q[0]);
+  const P nv[3] = {mul2(q[1], nir), mul2(q[2], nir), mul2(q[3], nir)};
+  const P* b = q + 5;
+  const P bd2 = mul2(b[D], b[D]);
+  const P B2 = fma2(b[B], b[B], fma2(b[A], b[A], bd2));
+  const P nSv = fma2(q[3], nv[2], fma2(q[2], nv[1], mul2(q[1], nv[0])));
+  const P pr = mul2(P(gamma - T(1)), fma2(P(T(0.5)), sub2(nSv, B2), q[4]));
+  const P pt = fma2(P(T(0.5)), B2, pr);
+  const P nvB = fma2(nv[2], b[2], fma2(nv[1], b[1], mul2(nv[0], b[0])));
+  const P nb = minus2(b[D]);
+  const P Sd = q[1 + D];
+  // signal speed |v_d| + c_fast
+  const P na2 = mul2(mul2(P(gamma), pr), nir);
+  const P ns = fma2(B2, nir, na2);
+  const P disc = fma2(mul2(P(T(-4)), na2), mul2(bd2, nir), mul2(ns, ns));
+  const P cf = sqrt2(mul2(P(T(0.5)), sub2(sqrt2(pos2(disc)), ns)));
+  const T S = larger(fabs(nv[D].x) + cf.x, fabs(nv[D].y) + cf.y);
+  auto out = [&](int f, P nf) { F[f] = fma(-S, q[f].y - q[f].x, -nf.x - nf.y); };
+  F[0] = fma(-S, q[0].y - q[0].x, Sd.x + Sd.y);
+  out(1 + D, sub2(fma2(Sd, nv[D], bd2), pt));
+  out(1 + A, fma2(b[D], b[A], mul2(Sd, nv[A])));
+  out(1 + B, fma2(b[D], b[B], mul2(Sd, nv[B])));
+  out(4, fma2(nb, nvB, mul2(add2(q[4], pt), nv[D])));
+  F[5 + D] = fma(-S, b[D].y - b[D].x, T(0));
+  out(5 + A, fma2(nb, nv[A], mul2(nv[D], b[A])));
+  out(5 + B, fma2(nb, nv[B], mul2(nv[D], b[B])));
+}
+
+}  // namespace sf
