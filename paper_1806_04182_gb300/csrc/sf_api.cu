@@ -214,18 +214,24 @@ namespace {
 // the stage kernels themselves use.
 constexpr long long kMaxSelftestCycles = 2000000000LL;
 
-// One warp waits on an mbarrier that nothing ever arrives on, through the
-// same bounded wait the TMA-staged kernels use; the wait gives up after
-// `limit` cycles and the kernel records ST_TIMEOUT.
+// One warp waits on an mbarrier that nothing ever arrives on, through the two
+// bounded waits that the TMA-staged kernels use (per thread, and per warp),
+// each for half of `limit` cycles; the kernel records ST_TIMEOUT once both
+// have given up.
 __global__ void wait_selftest_kernel(long long limit, unsigned int* status) {
   __shared__ uint64_t bar;
+  __shared__ unsigned gaveup;
   if (threadIdx.x == 0) {
+    gaveup = 0u;
     mbar_init(&bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
-  const bool ok = mbar_wait(&bar, 0, limit);
-  if (!ok && threadIdx.x == 0) atomicOr(status, ST_TIMEOUT);
+  const unsigned half = (unsigned)((limit + 1) / 2);
+  const bool ok = mbar_wait(&bar, 0, half);
+  __syncwarp();
+  mbar_wait_warp(&bar, 0, half, &gaveup);
+  if (!ok && threadIdx.x == 0 && *reinterpret_cast<volatile unsigned*>(&gaveup)) atomicOr(status, ST_TIMEOUT);
 }
 
 }  // namespace

@@ -109,8 +109,9 @@ struct sf_batch {
   std::vector<char> pair;  // patch q goes to the two-point CCZ4 kernel (takes precedence)
   void* d_pmaps = nullptr;   // its tensor maps, 6 per patch
   void* d_pcoefs = nullptr;  // its stencil weights, one block per patch
-  TmaTile* d_ptiles = nullptr;  // its 32 x 16 tiles
+  TmaTile* d_ptiles = nullptr;  // its tiles, those of shape 0, then of shape 1
   int npair = 0;                // two-point tiles
+  int nwide = 0;                // of which the first nwide are of shape 0
   void* d_maps = nullptr; // tensor maps, 3 per patch (u_n, u_stage, u_next roles)
   TmaTile* d_tiles = nullptr;   // 32 x 12 tiles, then 16 x 24 tiles
   int ntiles = 0;               // all TMA tiles
@@ -195,15 +196,15 @@ sf_status build_items(sf_batch* b, int only_class) {
 
 // Tensor maps, stencil weights and tile lists of the patches served by the
 // two-point CCZ4 kernel (double-word islands, the one-float row offset
-// layout): 32 x 16 tiles of every plane, overhanging the patch where its
-// size is not a multiple.
+// layout), each patch in tiles of its shape, overhanging it where its size is
+// not a multiple.
 sf_status build_pair(sf_batch* b) {
   b->pair.assign(b->npatch, 0);
-  b->npair = 0;
+  b->npair = b->nwide = 0;
   if (b->precision != SF_FP32_BULK_DW) return SF_OK;
   const size_t cb = z4_pair_coef_bytes();
   std::vector<unsigned char> maps((size_t)6 * b->npatch * kTmaMapBytes, 0), coefs(cb * b->npatch, 0);
-  std::vector<TmaTile> tiles;
+  std::vector<TmaTile> lists[2];
   for (int q = 0; q < b->npatch; ++q) {
     const sf_patch& p = b->patches[q];
     if (!z4_pair_batch_eligible(b->prm, p)) continue;
@@ -211,10 +212,15 @@ sf_status build_pair(sf_batch* b) {
     sf_status e = encode_z4_pair_batch(maps.data() + (size_t)6 * q * kTmaMapBytes, coefs.data() + cb * q,
                                        b->prm, p);
     if (e) return e;
-    for (int z = 0; z < p.n[2]; ++z)
-      for (int y = 0; y < p.n[1]; y += kPairTileY)
-        for (int x = 0; x < p.n[0]; x += kPairTileX) tiles.push_back(TmaTile{q, x, y, z});
+    const int w = z4_pair_shape(p);
+    const int* t = kPairShapes[w];
+    for (int z = 0; z < p.n[2]; z += t[2])
+      for (int y = 0; y < p.n[1]; y += t[1])
+        for (int x = 0; x < p.n[0]; x += t[0]) lists[w].push_back(TmaTile{q, x, y, z});
   }
+  std::vector<TmaTile>& tiles = lists[0];
+  b->nwide = (int)tiles.size();
+  tiles.insert(tiles.end(), lists[1].begin(), lists[1].end());
   b->npair = (int)tiles.size();
   if (tiles.empty()) return SF_OK;
   if (cudaMalloc(&b->d_pmaps, maps.size()) != cudaSuccess ||
@@ -304,7 +310,7 @@ sf_status launch_stage(sf_batch* b, int stage, cudaStream_t st, unsigned int* st
         static_cast<const PatchArgs<float>*>(b->d_args) + (size_t)stage * b->npatch;
     const StageArgs sa = batch_stage_args(b, stage, status);
     sf_status e = launch_z4_pair_batch(b->prm, b->d_pmaps, role[stage], fargs, b->d_pcoefs,
-                                       b->d_ptiles, b->npair, sa, st);
+                                       b->d_ptiles, b->npair, b->nwide, sa, st);
     const int n32 = b->ntiles - b->ntiles16;
     if (!e)
       e = launch_z4_tma_batch(b->prm, b->precision, b->d_maps, role[stage], fargs, b->d_tiles, n32,

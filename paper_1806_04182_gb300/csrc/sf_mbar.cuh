@@ -18,25 +18,72 @@ __device__ __forceinline__ void mbar_init(uint64_t* b, unsigned count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(saddr(b)), "r"(count) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_try(uint64_t* b, unsigned parity) {
+// Wait for the phase with the given parity, for at most `limit` clock cycles
+// (less than 2^32); false if it gave up.  Nine instructions: the stage
+// kernels inline some fifty waits each, and their code only just fits the
+// 128 KB from which an SM can stream instructions (see sf_z4_pair.cuh).
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity, unsigned limit) {
   unsigned ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      "{\n .reg .pred p;\n .reg .b32 t0, t;\n"
+      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " @p bra DONE;\n"
+      " mov.u32 t0, %%clock;\n"
+      "AGAIN:\n"
+      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " @p bra DONE;\n"
+      " mov.u32 t, %%clock;\n"
+      " sub.u32 t, t, t0;\n"
+      " setp.lt.u32 p, t, %3;\n"
+      " @p bra AGAIN;\n"
+      "DONE:\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
-      : "r"(saddr(b)), "r"(parity)
+      : "r"(saddr(b)), "r"(parity), "r"(limit)
       : "memory");
   return ok != 0;
 }
 
-// Wait for the phase with the given parity, for at most `limit` clock
-// cycles; false if it gave up.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, unsigned parity, long long limit) {
-  if (mbar_try(b, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try(b, parity))
-    if (clock64() - t0 > limit) return false;
-  return true;
+// The same for a converged warp, without a result: every lane waits, and the
+// branches are uniform (on a vote).  A wait that runs past the limit sets the
+// shared word *gaveup; once it is set, no wait of the CTA spins any more.  The
+// hot path is three instructions.
+__device__ __forceinline__ void mbar_wait_warp(uint64_t* b, unsigned parity, unsigned limit,
+                                               unsigned* gaveup) {
+  asm volatile(
+      "{\n .reg .pred p, q;\n .reg .b32 t0, t, g;\n"
+      " mov.u32 t0, 0;\n"
+      "AGAIN:\n"
+      " mbarrier.try_wait.parity.shared::cta.b64 p, [%0], %1;\n"
+      " vote.sync.all.pred p, p, 0xffffffff;\n"
+      " @p bra.uni DONE;\n"
+      " ld.volatile.shared.u32 g, [%3];\n"
+      " mov.u32 t, %%clock;\n"
+      " setp.eq.u32 q, t0, 0;\n"
+      " @q or.b32 t0, t, 1;\n"
+      " sub.u32 t, t, t0;\n"
+      " setp.gt.s32 q, t, %2;\n"
+      " setp.ne.or.u32 q, g, 0, q;\n"
+      " vote.sync.any.pred q, q, 0xffffffff;\n"
+      " @!q bra.uni AGAIN;\n"
+      " st.volatile.shared.u32 [%3], 1;\n"
+      "DONE:\n}\n" ::"r"(saddr(b)), "r"(parity), "r"(limit), "r"(saddr(gaveup))
+      : "memory");
+}
+
+// One lane of a converged warp (the same every time).
+__device__ __forceinline__ bool elect_one() {
+  unsigned r;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(r));
+  return r != 0;
+}
+
+// One arrival for a converged warp.
+__device__ __forceinline__ void mbar_arrive_warp(uint64_t* b) {
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n"
+      " @p mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n" ::"r"(saddr(b))
+      : "memory");
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* b) {

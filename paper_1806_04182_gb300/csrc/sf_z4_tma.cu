@@ -49,7 +49,7 @@ namespace {
 // end).
 constexpr int TX = 40, TZ = 7;
 constexpr int kSY = 104, kSZ = 104 * 102;         // global strides of the padded 96^3 layout
-constexpr long long kWaitCycles = 2000000000LL;   // ~1 s at GB300 clocks
+constexpr unsigned kWaitCycles = 2000000000u;   // ~1 s at GB300 clocks
 
 template <int BY, int KS, int XP = 32>
 struct Cfg {
@@ -83,8 +83,11 @@ static_assert(kTmaTileX16 == 16 && kTmaTileY16 == kBY16, "batch narrow tiles are
 // Order in which z4_cell opens the fields' stencils (cross, then the mixed
 // derivatives of the same field).  Without the Gamma-driver (shift frozen)
 // the last three are not used.
-__constant__ signed char kFieldSeq[25] = {19, 20, 21, 1, 2, 3, 4, 5, 6, 14, 15, 16, 0,
-                                          18, 7, 17, 8, 9, 10, 11, 12, 13, 22, 23, 24};
+__device__ __forceinline__ constexpr int tma_field(int use) {
+  constexpr signed char seq[25] = {19, 20, 21, 1, 2, 3, 4, 5, 6, 14, 15, 16, 0,
+                                   18, 7, 17, 8, 9, 10, 11, 12, 13, 22, 23, 24};
+  return seq[use];
+}
 
 __device__ __forceinline__ void tma_load_4d(float* dst, const CUtensorMap* map, int x, int y, int z,
                                             int f, uint64_t* bar) {
@@ -122,19 +125,14 @@ struct TmaSrc {
   __device__ __forceinline__ float ld(const float* q) const { return *q; }
   __device__ __forceinline__ float centre(int f) const { return __ldg(u + f * F); }
 
-  __device__ __forceinline__ void fail() {
-    if (!dead) atomicOr(status, ST_TIMEOUT);
-    dead = true;
-  }
-
   // leader: load field use j into its slot once the previous occupant
   // (use j - kSlots) has been released by every warp
   __device__ __forceinline__ void issue(int j) {
     const int sl = j % kSlots;
-    if (j >= kSlots && !dead && !mbar_wait(&empty[sl], ((j / kSlots) - 1) & 1, kWaitCycles)) fail();
+    if (j >= kSlots && !dead) dead = !mbar_wait(&empty[sl], ((j / kSlots) - 1) & 1, kWaitCycles);
     if (dead) return;
     mbar_expect(&full[sl], kBoxBytes);
-    tma_load_4d(tiles + sl * kSlotFloats, map, gx, gy, gz, kFieldSeq[j], &full[sl]);
+    tma_load_4d(tiles + sl * kSlotFloats, map, gx, gy, gz, tma_field(j), &full[sl]);
     issued = j + 1;
   }
 
@@ -151,12 +149,13 @@ struct TmaSrc {
       if (lane0) mbar_arrive(&empty[(i - 1) % kSlots]);
     }
     cur = i % kSlots;
-    if (!dead && !mbar_wait(&full[cur], (i / kSlots) & 1, kWaitCycles)) fail();
+    if (!dead) dead = !mbar_wait(&full[cur], (i / kSlots) & 1, kWaitCycles);
   }
 
   // the leader's warp consumed every load it issued unless a wait gave up;
   // then it waits (bounded) for the loads still in flight before exiting
   __device__ __forceinline__ void finish() {
+    if (dead) atomicOr(status, ST_TIMEOUT);
     if (leader && dead)
       for (int j = use; j < issued; ++j) mbar_wait(&full[j % kSlots], (j / kSlots) & 1, kWaitCycles);
   }
