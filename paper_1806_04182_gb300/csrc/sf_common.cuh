@@ -40,7 +40,8 @@ struct PatchArgs {
   // kernels that evaluate two directions at once (sf_pair.cuh): entry k of
   // direction d is cst[k][d]; pairs (x, y) are 8-byte aligned.
   //   0: 1/(12 dx)    1: 8/(12 dx)                          (D_d)
-  //   2: s   3: 15 s   4: -6 s   5: -20 s,  s = sigma/(64 dx)  (KO)
+  //   2: s   3: 15 s   4: -6 s   5: -20 s,  s = sigma/(64 dx)  (KO);
+  //   cst[5].v[3]: the sum of -20 s over the directions
   //   6: 16 e   7: -e   8: -30 e,  e = 1/(12 dx^2)            (D_dd)
   // and mixed: cmx[k] = (w, 8 w, 64 w)[k] with w = 1/(144 dx_a dx_b) for
   // (xy, xz) as a pair and yz alone.
@@ -288,6 +289,11 @@ PatchArgs<T> make_args(const sf_params& prm, const sf_patch& p, int stage, int n
     for (int k = 0; k < 9; ++k) a.cst[k].v[d] = T(w[k]);
   }
   for (int k = 0; k < 9; ++k) a.cst[k].v[3] = T(0);
+  {  // the KO weight of the centre summed over the directions
+    double kc = 0.0;
+    for (int d = 0; d < 3; ++d) kc += -20.0 * prm.sigma_ko / (64.0 * p.dx[d]);
+    a.cst[5].v[3] = T(kc);
+  }
   {
     const double wxy = 1.0 / (144.0 * p.dx[0] * p.dx[1]), wxz = 1.0 / (144.0 * p.dx[0] * p.dx[2]),
                  wyz = 1.0 / (144.0 * p.dx[1] * p.dx[2]);
