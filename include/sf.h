@@ -174,6 +174,19 @@ typedef struct {
   void* kahan;
 } sf_state;
 
+/*
+ * nsteps full RK steps of one patch whose state stays on the device: the
+ * stages of sf_substep (adjoint != 0: of sf_adjoint_substep) in the buffer
+ * roles u -> s1 -> s2 -> s1 -> u for RK4, u -> s1 -> s2 -> u for SSP-RK3, one
+ * launch per stage, enqueued by one call.  geom: n, ghost, dx, strides, dt,
+ * system, precision and cfl_rate (set by the last stage of every step; not
+ * with adjoint); its other pointers are ignored.  u must have valid ghosts.
+ * Errors: those of sf_substep for any stage, nsteps < 0, NULL arguments,
+ * adjoint steps that are not RK4; nothing is enqueued then.
+ */
+sf_status sf_steps(const sf_params* prm, const sf_patch* geom, const sf_state* state,
+                   int32_t nsteps, int32_t adjoint, void* stream);
+
 /* sf_step_host flag: zero the Kahan compensation of the slot at every upload. */
 #define SF_HOST_RESET_KAHAN 1u
 /* sf_step_host flag: host images are the interior only (sf_interior_span

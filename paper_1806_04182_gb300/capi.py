@@ -22,7 +22,7 @@ SF_GHOSTS_NONE, SF_GHOSTS_PERIODIC = 0, 1
 STATUS_NAMES = {0: "SF_OK", 1: "SF_EINVAL", 2: "SF_ENOTSUP", 3: "SF_ECUDA", 4: "SF_ENONFINITE",
                 5: "SF_ETIMEOUT"}
 
-EXPORTS = ["sf_nfields", "sf_substep", "sf_rhs", "sf_fill_ghosts_periodic", "sf_mhd_max_rate",
+EXPORTS = ["sf_nfields", "sf_substep", "sf_steps", "sf_rhs", "sf_fill_ghosts_periodic", "sf_mhd_max_rate",
            "sf_adjoint_substep", "sf_gather", "sf_scatter_add", "sf_diagnostics",
            "sf_batch_create", "sf_batch_substep", "sf_batch_tune", "sf_batch_capture",
            "sf_batch_launch", "sf_batch_launches_per_step", "sf_batch_destroy",
@@ -145,6 +145,7 @@ def lib() -> ctypes.CDLL:
         L.sf_nfields.restype = i32
         L.sf_substep.argtypes = [P(sf_params), P(sf_patch), i32, i32, vp]
         L.sf_rhs.argtypes = [P(sf_params), P(sf_patch), vp, vp]
+        L.sf_steps.argtypes = [P(sf_params), P(sf_patch), P(sf_state), i32, i32, vp]
         L.sf_fill_ghosts_periodic.argtypes = [P(sf_patch), vp, i32, vp]
         L.sf_mhd_max_rate.argtypes = [P(sf_params), P(sf_patch), vp, vp, vp]
         L.sf_adjoint_substep.argtypes = [P(sf_params), P(sf_patch), i32, i32, vp]
@@ -188,7 +189,7 @@ def lib() -> ctypes.CDLL:
                      "sf_batch_launch", "sf_batch_destroy", "sf_get_device_status",
                      "sf_batch_substep_static", "sf_copy_boxes", "sf_prolong",
                      "sf_batch_set_halo", "sf_selftest_wait_timeout", "sf_step_host",
-                     "sf_batch_tuned"):
+                     "sf_batch_tuned", "sf_steps"):
             getattr(L, name).restype = ctypes.c_int
         _lib = L
     return _lib
@@ -236,6 +237,13 @@ def sf_nfields(system: int) -> int:
 def sf_substep(prm: sf_params, patches, stage: int, stream: int = 0) -> None:
     arr, n = _patches(patches)
     _check(lib().sf_substep(ctypes.byref(prm), arr, n, stage, stream), "sf_substep")
+
+
+def sf_steps(prm: sf_params, geom: sf_patch, state: sf_state, nsteps: int, adjoint: bool = False,
+             stream: int = 0) -> None:
+    """nsteps full RK steps of a device-resident patch state, enqueued by one call."""
+    _check(lib().sf_steps(ctypes.byref(prm), ctypes.byref(geom), ctypes.byref(state), nsteps,
+                          1 if adjoint else 0, stream), "sf_steps")
 
 
 def sf_adjoint_substep(prm: sf_params, patches, stage: int, stream: int = 0) -> None:

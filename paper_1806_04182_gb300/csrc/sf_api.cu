@@ -322,6 +322,37 @@ sf_status sf_adjoint_substep(const sf_params* prm, const sf_patch* adj, int32_t 
   return SF_OK;
 }
 
+sf_status sf_steps(const sf_params* prm, const sf_patch* geom, const sf_state* state,
+                   int32_t nsteps, int32_t adjoint, void* stream) {
+  t_err[0] = 0;
+  if (!prm || !geom || !state || nsteps < 0) return set_error(SF_EINVAL, "NULL argument or nsteps < 0");
+  if (prm->rk != SF_RK4 && prm->rk != SF_SSPRK3) return set_error(SF_EINVAL, "unknown rk %d", prm->rk);
+  if (adjoint && geom->system != SF_WAVE)
+    return set_error(SF_ENOTSUP, "adjoint steps exist for SF_WAVE only");
+  if (adjoint && prm->rk != SF_RK4) return set_error(SF_EINVAL, "adjoint steps are RK4 steps");
+  const int ns = prm->rk == SF_RK4 ? 4 : 3;
+  void* us[4] = {state->u, state->s1, state->s2, state->s1};
+  void* nx[4] = {state->s1, state->s2, ns == 4 ? state->s1 : state->u, state->u};
+  sf_patch p[4];
+  StageArgs s[4];
+  for (int q = 0; q < ns; ++q) {
+    p[q] = *geom;
+    normalise_strides(p[q], sf_nfields(p[q].system));
+    p[q].u_stage = us[q];
+    p[q].u_n = state->u;
+    p[q].u_next = nx[q];
+    p[q].acc = state->acc;
+    p[q].kahan = state->kahan;
+    if (adjoint) p[q].cfl_rate = nullptr;
+    if (sf_status e = check_patch(prm, p[q], 1, q)) return e;
+    s[q] = stage_args(*prm, p[q], q, 0);
+  }
+  for (int k = 0; k < nsteps; ++k)
+    for (int q = 0; q < ns; ++q)
+      if (sf_status e = dispatch(*prm, p[q], s[q], q, nullptr, adjoint != 0, (cudaStream_t)stream)) return e;
+  return SF_OK;
+}
+
 sf_status sf_rhs(const sf_params* prm, const sf_patch* patch, void* rhs_out, void* stream) {
   t_err[0] = 0;
   if (!patch || !rhs_out) return set_error(SF_EINVAL, "patch or rhs_out NULL");

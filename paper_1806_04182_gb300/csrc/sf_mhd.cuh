@@ -126,8 +126,6 @@ __device__ __forceinline__ R2 pos2(R2 x) {
 }
 __device__ __forceinline__ F2 abs2(F2 x) { return F2(fabsf(x.x), fabsf(x.y)); }
 __device__ __forceinline__ R2 abs2(R2 x) { return R2(fabs(x.x), fabs(x.y)); }
-__device__ __forceinline__ F2 minus2(F2 x) { return mul2(x, F2(-1.0f)); }
-__device__ __forceinline__ R2 minus2(R2 x) { return neg2(x); }
 // the larger of two non-negative values; double: as integers (their bits are
 // ordered alike, NaN above all)
 __device__ __forceinline__ float larger(float a, float b) { return a > b ? a : b; }
@@ -242,7 +240,7 @@ __device__ __forceinline__ void weno_edges(const P* w, T eps, const MhdCoef<T>& 
     const P q0 = mul2(p0, d2), q1 = mul2(p1, d1), two(T(2));
     P ir, il;
     half_recips<VAR>(fma2(two, p0, p1), fma2(two, p1, p0), ir, il);
-    er = fma2(fma2(P(T(-2)), q0, minus2(q1)), ir, w[2]);
+    er = fma2(fma2(P(T(-2)), q0, neg2(q1)), ir, w[2]);
     el = fma2(fma2(two, q1, q0), il, w[2]);
     return;
   }
@@ -286,7 +284,7 @@ __device__ __forceinline__ void llf_flux2(const P* q, T gamma, T* F) {
   const P pr = mul2(P(gamma - T(1)), fma2(P(T(0.5)), sub2(nSv, B2), q[4]));
   const P pt = fma2(P(T(0.5)), B2, pr);
   const P nvB = fma2(nv[2], b[2], fma2(nv[1], b[1], mul2(nv[0], b[0])));
-  const P nb = minus2(b[D]);
+  const P nb = neg2(b[D]);
   const P Sd = q[1 + D];
   // signal speed |v_d| + c_fast
   const P na2 = mul2(mul2(P(gamma), pr), nir);

@@ -12,6 +12,7 @@ SSP-RK3: stage 0: A -> B, 1: B -> C, 2: C -> A.
 from __future__ import annotations
 
 import json
+import struct
 
 import numpy as np
 import torch
@@ -190,12 +191,25 @@ class PatchState:
         capi.sf_substep(self.prm, self.stage_patch(s), s, _stream_handle(stream))
         return self.roles(s)[1]
 
+    # sf_patch and sf_state as bytes, in the order of their fields (one pack call
+    # instead of an attribute assignment per field: a step of a small patch
+    # takes less time on the GPU than its descriptors took to fill)
+    _GEOM = struct.Struct("=4i4d2i3q6Q")
+    _STATE = struct.Struct("=5Q")
+
+    def _steps(self, nsteps: int, h: int, adjoint: bool = False, rate: int = 0) -> None:
+        g = capi.sf_patch.from_buffer_copy(self._GEOM.pack(
+            *self.n, self.g, *self.dx, self.dt, self.system, self.precision, *self.strides,
+            0, 0, 0, 0, 0, rate))
+        s = capi.sf_state.from_buffer_copy(self._STATE.pack(
+            self.ptr(self.A), self.ptr(self.B), self.ptr(self.C),
+            self.ptr(self.D) if self.D is not None else 0,
+            self.ptr(self.E) if self.E is not None else 0))
+        capi.sf_steps(self.prm, g, s, nsteps, adjoint, h)
+
     def step(self, nsteps: int = 1, stream=None) -> None:
         self._rate = None
-        h = _stream_handle(stream)
-        for _ in range(nsteps):
-            for s in range(self.nstages):
-                capi.sf_substep(self.prm, self.stage_patch(s), s, h)
+        self._steps(nsteps, _stream_handle(stream))
 
     def step_cfl(self, nsteps: int = 1, cfl: float = 0.3, stream=None) -> list[float]:
         """MHD steps with dt = cfl / rate, the rate of U^n coming from the
@@ -213,19 +227,12 @@ class PatchState:
             r = rate.item()
             rates.append(r)
             self.dt = cfl / r
-            for s in range(self.nstages):
-                p = self.stage_patch(s)
-                if s == self.nstages - 1:
-                    p.cfl_rate = rate.data_ptr()
-                capi.sf_substep(self.prm, p, s, h)
+            self._steps(1, h, rate=rate.data_ptr())
         return rates
 
     def adjoint_step(self, nsteps: int = 1, stream=None) -> None:
         """RK4 steps of the transposed wave operator on A (adjoint fields)."""
-        h = _stream_handle(stream)
-        for _ in range(nsteps):
-            for s in range(4):
-                capi.sf_adjoint_substep(self.prm, self.stage_patch(s), s, h)
+        self._steps(nsteps, _stream_handle(stream), adjoint=True)
 
     def rhs(self, array: torch.Tensor | None = None, stream=None) -> torch.Tensor:
         """(L + Q_d)(array) on the interior, shape (nf, nz, ny, nx)."""
