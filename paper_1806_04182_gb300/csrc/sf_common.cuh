@@ -260,6 +260,34 @@ struct Launch {
   dim3 grid, block;
 };
 
+// Programmatic stream serialization: the launch of a kernel that waits for its
+// predecessor itself overlaps the predecessor's end (its blocks are placed when
+// the last of the predecessor's has exited, before its memory is flushed).
+// Every kernel launched by launch_after() calls wait_predecessor() before it
+// reads or writes global memory; without an explicit trigger, so that no
+// waiting block takes a place from a running one (triggering at the start made
+// FP64 wave stages of 24^3 twice as slow).  Chains of small stages gain most:
+// 16^3 wave stage 6.2 -> 3.3 us.
+__device__ __forceinline__ void wait_predecessor() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename... Args>
+void launch_after(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                  Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Host-side construction of PatchArgs from the ABI structs.
 template <typename T>
 PatchArgs<T> make_args(const sf_params& prm, const sf_patch& p, int stage, int nf,

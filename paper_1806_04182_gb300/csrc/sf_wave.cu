@@ -6,7 +6,8 @@
 namespace sf {
 
 template <typename T, bool ADJ>
-__global__ void __launch_bounds__(128) wave_stage_kernel(PatchArgs<T> a, StageArgs s) {
+__global__ void __launch_bounds__(128, 4) wave_stage_kernel(PatchArgs<T> a, StageArgs s) {
+  wait_predecessor();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -14,10 +15,39 @@ __global__ void __launch_bounds__(128) wave_stage_kernel(PatchArgs<T> a, StageAr
   const int g = a.g;
   const long long c = (long long)(k + g) * a.sz + (long long)(j + g) * a.sy + (i + g);
   T v[5], r[5];
+  if (s.mode == 1) {
+    wave_point<T, ADJ>(a, a.us + c, v, r);
+#pragma unroll
+    for (int f = 0; f < 5; ++f) a.nx[f * a.ninterior + ((long long)k * a.n[1] + j) * a.n[0] + i] = r[f];
+    return;
+  }
+  // The RK inputs are read first, beside the stencils: read field by field in
+  // the stage write, behind the stores of the field before, they made five
+  // round trips to memory one after another (a 16^3 stage is nothing but
+  // latency: 8.2 us, then 6.2; the bound on registers lets the compiler keep
+  // more loads in flight).
+  T un[5], acc[5], kh[5];
+  const bool rk4 = s.rk == SF_RK4;
+#pragma unroll
+  for (int f = 0; f < 5; ++f) {
+    const long long o = f * a.sf + c;
+    un[f] = s.un_alias ? T(0) : a.un[o];
+    acc[f] = (rk4 && s.stage > 0) ? a.acc[o] : T(0);
+    kh[f] = (rk4 && s.stage == 3 && s.kahan) ? a.kh[o] : T(0);
+  }
   wave_point<T, ADJ>(a, a.us + c, v, r);
   const Images im = ghost_images(a, s, i, j, k);
 #pragma unroll
-  for (int f = 0; f < 5; ++f) write_field(a, s, im, f, c, i, j, k, v[f], r[f]);
+  for (int f = 0; f < 5; ++f) {
+    const long long o = f * a.sf + c;
+    r[f] = stage_combine(a, s, o, v[f], un[f], acc[f], kh[f], r[f]);
+    a.nx[o] = r[f];
+    if (s.check_finite && !finite_(r[f])) atomicOr(s.status, ST_NONFINITE);
+  }
+  if (im.mask) {
+#pragma unroll
+    for (int f = 0; f < 5; ++f) store_images(a, im, f * a.sf + c, r[f]);
+  }
 }
 
 // float: a block of 32 x 8 columns marches mz planes in z.  Planes of the
@@ -84,6 +114,7 @@ __global__ void __launch_bounds__(kMarchX * kMarchY, 3)
     const int cx = min(x0 - 3 + t % CW, a.n[0] + 2), cy = min(y0 - 3 + t / CW, a.n[1] + 2);
     so[e] = (k0 + g) * sz + (cy + g) * sy + (cx + g);
   }
+  wait_predecessor();
   const unsigned ring0 = (unsigned)__cvta_generic_to_shared(ring) + tid * 4;
   int left = k1 + 3 - k0;  // planes still to be staged
   int ws = 0;              // slot they go to, in elements
@@ -240,16 +271,13 @@ static sf_status launch(const sf_params& prm, const sf_patch& p, const StageArgs
                                       : (form == 1 ? wave_march_kernel<true, 1> : wave_march_kernel<true, 2>))
                          : (form == 0 ? wave_march_kernel<false, 0>
                                       : (form == 1 ? wave_march_kernel<false, 1> : wave_march_kernel<false, 2>));
-      kernel<<<grid, dim3(kMarchX, kMarchY), kMarchSmem, st>>>(a, s, mz);
+      launch_after(kernel, grid, dim3(kMarchX, kMarchY), kMarchSmem, st, a, s, mz);
       return after_launch("wave_march_kernel");
     }
   }
   dim3 block(32, 4, 1);
   dim3 grid((p.n[0] + 31) / 32, (p.n[1] + 3) / 4, p.n[2]);
-  if (adj)
-    wave_stage_kernel<T, true><<<grid, block, 0, st>>>(a, s);
-  else
-    wave_stage_kernel<T, false><<<grid, block, 0, st>>>(a, s);
+  launch_after(adj ? wave_stage_kernel<T, true> : wave_stage_kernel<T, false>, grid, block, 0, st, a, s);
   return after_launch("wave_stage_kernel");
 }
 
