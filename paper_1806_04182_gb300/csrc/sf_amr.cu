@@ -44,6 +44,7 @@ constexpr int kCopyIlp = 8;
 
 template <typename T>
 __global__ void __launch_bounds__(256) copy_boxes_kernel(BoxBatch bb) {
+  wait_predecessor();
   int lo = 0, hi = bb.n - 1;  // first box with end > blockIdx.x
   while (lo < hi) {
     const int mid = (lo + hi) / 2;
@@ -327,6 +328,7 @@ __device__ __forceinline__ void prolong_kind(const Combo<T>& cb, const ProlongAr
 template <typename T, int NS>
 __global__ void __launch_bounds__(kProlongThreads) prolong_kernel(Combo<T> cb, ProlongArgs p) {
   extern __shared__ __align__(16) unsigned char psm_raw[];
+  wait_predecessor();
   // the CTA's box, tile and field (one field per CTA, field slowest)
   int bi = 0;
   while (bi + 1 < p.nbox && (int)blockIdx.x >= p.tiles_end[bi]) ++bi;
@@ -493,9 +495,9 @@ extern "C" sf_status sf_copy_boxes(const sf_box_copy* boxes, int32_t nbox, int32
     }
     if (bb.n == 0) continue;
     if (precision == SF_FP64)
-      copy_boxes_kernel<double><<<blocks, 256, 0, st>>>(bb);
+      launch_after(copy_boxes_kernel<double>, blocks, 256, 0, st, bb);
     else
-      copy_boxes_kernel<float><<<blocks, 256, 0, st>>>(bb);
+      launch_after(copy_boxes_kernel<float>, blocks, 256, 0, st, bb);
     sf_status e = after_launch("copy_boxes_kernel");
     if (e) return e;
   }
@@ -606,8 +608,8 @@ static sf_status prolong_launch(const sf_patch* coarse, const void* const* array
         cudaFuncSetAttribute(prolong_kernel<double, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              prolong_smem_max<double>());
       });
-      prolong_kernel<double, NS><<<(unsigned)total, kProlongThreads, prolong_smem_bytes<double>(smem_elems),
-                                    st>>>(cb, a);
+      launch_after(prolong_kernel<double, NS>, (unsigned)total, kProlongThreads, prolong_smem_bytes<double>(smem_elems), st,
+                   cb, a);
     } else {
       Combo<float> cb;
       for (int m = 0; m < 5; ++m) cb.s[m] = m <= NS ? (const float*)arrays[m] : nullptr;
@@ -617,8 +619,8 @@ static sf_status prolong_launch(const sf_patch* coarse, const void* const* array
         cudaFuncSetAttribute(prolong_kernel<float, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              prolong_smem_max<float>());
       });
-      prolong_kernel<float, NS><<<(unsigned)total, kProlongThreads, prolong_smem_bytes<float>(smem_elems),
-                                   st>>>(cb, a);
+      launch_after(prolong_kernel<float, NS>, (unsigned)total, kProlongThreads, prolong_smem_bytes<float>(smem_elems), st,
+                   cb, a);
     }
     e = after_launch("prolong_kernel");
     if (e) return e;

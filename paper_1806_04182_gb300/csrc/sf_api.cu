@@ -112,6 +112,7 @@ sf_status check_patch(const sf_params* prm, const sf_patch& p, int need_stage_ar
 template <typename T>
 __global__ void __launch_bounds__(256) ghost_fill_kernel(T* u, int nx, int ny, int nz, int g,
                                                          long long sy, long long sz, long long sf) {
+  wait_predecessor();
   const unsigned X = nx + 2 * g, Y = ny + 2 * g, G2 = 2 * g;
   const unsigned s1 = G2 * X * Y, s2 = G2 * X * nz, total = s1 + s2 + G2 * ny * nz;
   T* uf = u + blockIdx.y * sf;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(256) ghost_fill_kernel(T* u, int nx, int ny, i
 template <typename T>
 __global__ void gather_kernel(const T* a, long long off, int nx, int ny, int g, long long sy,
                               long long sz, long long total, const int64_t* obs, int nobs, T* out) {
+  wait_predecessor();
   int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= nobs) return;
   long long lin = obs[o];
@@ -169,6 +171,7 @@ template <typename T>
 __global__ void scatter_add_kernel(T* a, long long off, int nx, int ny, int g, long long sy,
                                    long long sz, long long total, const int64_t* obs, int nobs,
                                    const T* vals) {
+  wait_predecessor();
   int o = blockIdx.x * blockDim.x + threadIdx.x;
   if (o >= nobs) return;
   long long lin = obs[o];
@@ -387,10 +390,10 @@ sf_status sf_fill_ghosts_periodic(const sf_patch* patch, void* array, int32_t nf
   if (gx > 1024) gx = 1024;
   const dim3 grid((unsigned)gx, (unsigned)nf);
   if (p.precision == SF_FP64)
-    ghost_fill_kernel<double><<<grid, 256, 0, (cudaStream_t)stream>>>(
+    launch_after(ghost_fill_kernel<double>, grid, 256, 0, (cudaStream_t)stream,
         (double*)array, p.n[0], p.n[1], p.n[2], p.ghost, p.sy, p.sz, p.sf);
   else
-    ghost_fill_kernel<float><<<grid, 256, 0, (cudaStream_t)stream>>>(
+    launch_after(ghost_fill_kernel<float>, grid, 256, 0, (cudaStream_t)stream,
         (float*)array, p.n[0], p.n[1], p.n[2], p.ghost, p.sy, p.sz, p.sf);
   return after_launch("ghost_fill_kernel");
 }
@@ -416,11 +419,11 @@ sf_status sf_gather(const sf_patch* patch, const void* array, int32_t field, con
   if (nobs == 0) return SF_OK;
   int blocks = (nobs + 127) / 128;
   if (p.precision == SF_FP64)
-    gather_kernel<double><<<blocks, 128, 0, (cudaStream_t)stream>>>(
+    launch_after(gather_kernel<double>, blocks, 128, 0, (cudaStream_t)stream,
         (const double*)array, field * p.sf, p.n[0], p.n[1], p.ghost, p.sy, p.sz,
         (long long)p.n[0] * p.n[1] * p.n[2], obs, nobs, (double*)out);
   else
-    gather_kernel<float><<<blocks, 128, 0, (cudaStream_t)stream>>>(
+    launch_after(gather_kernel<float>, blocks, 128, 0, (cudaStream_t)stream,
         (const float*)array, field * p.sf, p.n[0], p.n[1], p.ghost, p.sy, p.sz,
         (long long)p.n[0] * p.n[1] * p.n[2], obs, nobs, (float*)out);
   return after_launch("gather_kernel");
@@ -435,11 +438,11 @@ sf_status sf_scatter_add(const sf_patch* patch, void* array, int32_t field, cons
   if (nobs == 0) return SF_OK;
   int blocks = (nobs + 127) / 128;
   if (p.precision == SF_FP64)
-    scatter_add_kernel<double><<<blocks, 128, 0, (cudaStream_t)stream>>>(
+    launch_after(scatter_add_kernel<double>, blocks, 128, 0, (cudaStream_t)stream,
         (double*)array, field * p.sf, p.n[0], p.n[1], p.ghost, p.sy, p.sz,
         (long long)p.n[0] * p.n[1] * p.n[2], obs, nobs, (const double*)vals);
   else
-    scatter_add_kernel<float><<<blocks, 128, 0, (cudaStream_t)stream>>>(
+    launch_after(scatter_add_kernel<float>, blocks, 128, 0, (cudaStream_t)stream,
         (float*)array, field * p.sf, p.n[0], p.n[1], p.ghost, p.sy, p.sz,
         (long long)p.n[0] * p.n[1] * p.n[2], obs, nobs, (const float*)vals);
   return after_launch("scatter_add_kernel");

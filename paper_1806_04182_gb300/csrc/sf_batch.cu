@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2) batch_stage_kerne
                                                           const Item* __restrict__ items, int nitems,
                                                           unsigned int* counter, StageArgs s,
                                                           Z4Coef<T> zc) {
+  wait_predecessor();
   __shared__ int s_item;
   __shared__ T rbuf[25 * 128];  // parked CCZ4 right-hand sides (see write_fields)
   for (;;) {
@@ -335,11 +336,11 @@ sf_status launch_stage(sf_batch* b, int stage, cudaStream_t st, unsigned int* st
   const int grid = b->grid[b->precision];
   const StageArgs sa = batch_stage_args(b, stage, status);
   if (b->prm.lopsided)
-    batch_stage_kernel<T, H, true><<<grid, 128, 0, st>>>(args, b->d_sys, b->d_shape, b->d_items,
-                                                         b->nitems, b->d_counter, sa, zc);
+    launch_after(batch_stage_kernel<T, H, true>, grid, 128, 0, st, args, b->d_sys, b->d_shape, b->d_items,
+                 b->nitems, b->d_counter, sa, zc);
   else
-    batch_stage_kernel<T, H, false><<<grid, 128, 0, st>>>(args, b->d_sys, b->d_shape, b->d_items,
-                                                          b->nitems, b->d_counter, sa, zc);
+    launch_after(batch_stage_kernel<T, H, false>, grid, 128, 0, st, args, b->d_sys, b->d_shape, b->d_items,
+                 b->nitems, b->d_counter, sa, zc);
   return after_launch("batch_stage_kernel");
 }
 

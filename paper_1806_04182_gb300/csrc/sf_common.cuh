@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "../../include/sf.h"
 
 namespace sf {
@@ -272,9 +274,9 @@ __device__ __forceinline__ void wait_predecessor() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-template <typename... Args>
-void launch_after(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                  Args... args) {
+template <typename... Params, typename... Args>
+void launch_after(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                  Args&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -285,7 +287,7 @@ void launch_after(void (*kernel)(Args...), dim3 grid, dim3 block, size_t smem, c
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = 1;
-  cudaLaunchKernelEx(&cfg, kernel, args...);
+  cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
 // Host-side construction of PatchArgs from the ABI structs.

@@ -298,6 +298,7 @@ __global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
   constexpr bool ST = S::kStaged;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   S& sm = *reinterpret_cast<S*>(smem_raw);
+  wait_predecessor();
   const int tx = threadIdx.x, ty = threadIdx.y;
   const bool row = ty < MR;
   const int x0 = blockIdx.x * MX, y0 = blockIdx.y * MR;
@@ -560,6 +561,7 @@ template <typename T, int VAR>
 __global__ void __launch_bounds__(MX * SY)
     mhd_split_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, int mz) {
   __shared__ T fy[SY][MX][8];
+  wait_predecessor();
   __shared__ double s_rate[SY];
   const int tx = threadIdx.x, ty = threadIdx.y;
   double rate = 0.0;  // max signal rate of this thread's outputs (fused CFL reduction)
@@ -740,7 +742,7 @@ struct MhdInstance {
                      int mz, cudaStream_t st) {
     const dim3 block(MX, threads_y, 1);
     const dim3 grid((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y, (p.n[2] + mz - 1) / mz);
-    kernel()<<<grid, block, smem, st>>>(a, s, mc, mz);
+    launch_after(kernel(), grid, block, smem, st, a, s, mc, mz);
   }
 };
 

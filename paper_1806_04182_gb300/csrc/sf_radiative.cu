@@ -66,6 +66,7 @@ __device__ __forceinline__ void rad_d(const T* const (&p)[kFieldGroup], long lon
 
 template <typename T>
 __global__ void __launch_bounds__(256) radiative_kernel(PatchArgs<T> a, StageArgs s, RadArgs<T> ra) {
+  wait_predecessor();
   const unsigned g = (unsigned)a.g;
   const unsigned N0 = a.n[0] + 2 * g, N1 = a.n[1] + 2 * g;
   const unsigned zslab = 2 * g * N1 * N0;
@@ -163,7 +164,7 @@ sf_status launch(const sf_params& prm, const sf_patch& p, const StageArgs& s, in
   long long blocks = (ghosts + 255) / 256;
   if (blocks > 152 * 8) blocks = 152 * 8;
   const dim3 grid((unsigned)blocks, (unsigned)((ra.nf + kFieldGroup - 1) / kFieldGroup));
-  radiative_kernel<T><<<grid, 256, 0, st>>>(a, s, ra);
+  launch_after(radiative_kernel<T>, grid, 256, 0, st, a, s, ra);
   return after_launch("radiative_kernel");
 }
 

@@ -23,6 +23,7 @@ template <typename T, typename H, int SY, int SZ, bool LOP>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2)
     z4_stage_kernel(PatchArgs<T> a, StageArgs s, Z4Coef<T> zc) {
   __shared__ T rbuf[25 * 128];
+  wait_predecessor();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k = blockIdx.z;
@@ -46,11 +47,11 @@ static sf_status launch(const sf_params& prm, const sf_patch& p, const StageArgs
   dim3 block(32, 4, 1);
   dim3 grid((p.n[0] + 31) / 32, (p.n[1] + 3) / 4, p.n[2]);
   if (prm.lopsided)
-    z4_stage_kernel<T, H, 0, 0, true><<<grid, block, 0, st>>>(a, s, zc);
+    launch_after(z4_stage_kernel<T, H, 0, 0, true>, grid, block, 0, st, a, s, zc);
   else if (p.sy == 102 && p.sz == 102 * 102)
-    z4_stage_kernel<T, H, 102, 102 * 102, false><<<grid, block, 0, st>>>(a, s, zc);
+    launch_after(z4_stage_kernel<T, H, 102, 102 * 102, false>, grid, block, 0, st, a, s, zc);
   else
-    z4_stage_kernel<T, H, 0, 0, false><<<grid, block, 0, st>>>(a, s, zc);
+    launch_after(z4_stage_kernel<T, H, 0, 0, false>, grid, block, 0, st, a, s, zc);
   return after_launch("z4_stage_kernel");
 }
 

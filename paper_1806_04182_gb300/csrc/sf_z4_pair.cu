@@ -64,16 +64,16 @@ sf_status launch_pair(const sf_params& prm, const sf_patch& p, const StageArgs& 
   const dim3 grid(p.n[0] / C::BX, p.n[1] / C::BY, p.n[2]);
   switch (form) {
     case kRk4First:
-      z4_pair_kernel<H2, C, kRk4First><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_kernel<H2, C, kRk4First>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
       break;
     case kRk4Mid:
-      z4_pair_kernel<H2, C, kRk4Mid><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_kernel<H2, C, kRk4Mid>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
       break;
     case kRk4Last:
-      z4_pair_kernel<H2, C, kRk4Last><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_kernel<H2, C, kRk4Last>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
       break;
     default:
-      z4_pair_kernel<H2, C, kRkGeneric><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_kernel<H2, C, kRkGeneric>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
   }
   sf_status e = after_launch("z4_pair_kernel");
   // the RK4 forms write the x images themselves

@@ -620,6 +620,7 @@ __device__ __forceinline__ void pair_tile(const CUtensorMap* map, const CUtensor
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  wait_predecessor();
   __syncthreads();
   const int px = C::lane_x(threadIdx.x);
   const int lr = C::lane_row(threadIdx.y, threadIdx.x);  // row of the tile

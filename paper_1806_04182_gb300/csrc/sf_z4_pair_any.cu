@@ -54,6 +54,7 @@ __global__ void __launch_bounds__(32 * kPairWarps, 1)
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ PatchArgs<float> pa;
   __shared__ PairCoef pcs;
+  wait_predecessor();
   const TmaTile w = tl[blockIdx.x];
   {
     static_assert(sizeof(PatchArgs<float>) % 4 == 0 && sizeof(PairCoef) % 4 == 0, "word copy");
@@ -95,13 +96,13 @@ sf_status launch_any(const sf_params& prm, const sf_patch& p, const StageArgs& s
   const dim3 grid((p.n[0] + C::BX - 1) / C::BX, (p.n[1] + C::BY - 1) / C::BY, (p.n[2] + C::BZ - 1) / C::BZ);
   switch (form) {
     case kRk4First:
-      z4_pair_any_kernel<C, kRk4First><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_any_kernel<C, kRk4First>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
       break;
     case kRk4Mid:
-      z4_pair_any_kernel<C, kRk4Mid><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_any_kernel<C, kRk4Mid>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
       break;
     default:
-      z4_pair_any_kernel<C, kRk4Last><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc, pc, rk);
+      launch_after(z4_pair_any_kernel<C, kRk4Last>, grid, block, C::kSmemBytes, st, map, a, s, zc, pc, rk);
   }
   return after_launch("z4_pair_any_kernel");
 }
@@ -177,13 +178,13 @@ sf_status launch_z4_pair_batch(const sf_params& prm, const void* d_maps, int rol
   const dim3 block(32, kPairWarps, 1);
   switch (rk_form(s)) {
     case kRk4First:
-      z4_pair_batch_kernel<kRk4First><<<ntiles, block, smem, st>>>(maps, role, d_args, coefs, d_tiles, nwide, s, zc);
+      launch_after(z4_pair_batch_kernel<kRk4First>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
       break;
     case kRk4Mid:
-      z4_pair_batch_kernel<kRk4Mid><<<ntiles, block, smem, st>>>(maps, role, d_args, coefs, d_tiles, nwide, s, zc);
+      launch_after(z4_pair_batch_kernel<kRk4Mid>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
       break;
     case kRk4Last:
-      z4_pair_batch_kernel<kRk4Last><<<ntiles, block, smem, st>>>(maps, role, d_args, coefs, d_tiles, nwide, s, zc);
+      launch_after(z4_pair_batch_kernel<kRk4Last>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
       break;
     default:
       return set_error(SF_EINVAL, "batched two-point tiles need the RK4 Kahan forms");

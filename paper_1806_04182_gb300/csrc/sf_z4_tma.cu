@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(Cfg<BY, KS>::kThreads, Cfg<BY, KS>::kMinBlocks
   float* tiles = reinterpret_cast<float*>(smem);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + kSlots * C::kSlotFloats * 4);
   uint64_t* empty = full + kSlots;
+  wait_predecessor();
   const int tid = threadIdx.y * 32 + threadIdx.x;
   if (tid == 0) {
     for (int q = 0; q < kSlots; ++q) {
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(Cfg<kBY, kKS>::kThreads, 1)
     z4_tma_any_kernel(const __grid_constant__ CUtensorMap map, PatchArgs<float> a, StageArgs s,
                       Z4Coef<float> zc) {
   extern __shared__ __align__(128) unsigned char smem[];
+  wait_predecessor();
   init_ring(smem);
   __syncthreads();
   tma_tile_runtime<H, 32>(&map, a, s, zc, blockIdx.x * 32, blockIdx.y * kBY, blockIdx.z, smem);
@@ -310,6 +312,7 @@ __global__ void __launch_bounds__(Cfg<kBY, kKS>::kThreads, 1)
   using C = Cfg<kBY, kKS>;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ PatchArgs<float> pa;
+  wait_predecessor();
   const TmaTile w = tl[blockIdx.x];
   {
     static_assert(sizeof(PatchArgs<float>) % 4 == 0, "word copy");
@@ -365,7 +368,7 @@ sf_status launch_tma(const sf_params& prm, const sf_patch& p, const StageArgs& s
   const Z4Coef<float> zc = z4_coef<float>(prm);
   dim3 block(32, BY, 1);
   dim3 grid(p.n[0] / 32, p.n[1] / BY, p.n[2]);
-  z4_tma_kernel<H, BY, KS><<<grid, block, C::kSmemBytes, st>>>(map, a, s, zc);
+  launch_after(z4_tma_kernel<H, BY, KS>, grid, block, C::kSmemBytes, st, map, a, s, zc);
   return after_launch("z4_tma_kernel");
 }
 
@@ -432,8 +435,7 @@ sf_status launch_tma_batch(const sf_params& prm, const void* d_maps, int role,
                          C::kSmemBytes);
   });
   const Z4Coef<float> zc = z4_coef<float>(prm);
-  z4_tma_batch_kernel<H, XP><<<ntiles, dim3(32, kBY, 1), C::kSmemBytes, st>>>(
-      static_cast<const CUtensorMap*>(d_maps), role, d_args, d_tiles, s, zc);
+  launch_after(z4_tma_batch_kernel<H, XP>, ntiles, dim3(32, kBY, 1), C::kSmemBytes, st, static_cast<const CUtensorMap*>(d_maps), role, d_args, d_tiles, s, zc);
   return after_launch("z4_tma_batch_kernel");
 }
 }  // namespace
@@ -466,7 +468,7 @@ sf_status launch_tma_any(const sf_params& prm, const sf_patch& p, const StageArg
   PatchArgs<float> a = make_args<float>(prm, p, stage, 25, rhs_out);
   const Z4Coef<float> zc = z4_coef<float>(prm);
   dim3 grid((p.n[0] + 31) / 32, (p.n[1] + kBY - 1) / kBY, p.n[2]);
-  z4_tma_any_kernel<H><<<grid, dim3(32, kBY, 1), C::kSmemBytes, st>>>(
+  launch_after(z4_tma_any_kernel<H>, grid, dim3(32, kBY, 1), C::kSmemBytes, st, 
       *reinterpret_cast<const CUtensorMap*>(map), a, s, zc);
   return after_launch("z4_tma_any_kernel");
 }
