@@ -201,12 +201,40 @@ __device__ __forceinline__ void block_rate(double rate, double* s_rate, double* 
   }
 }
 
-template <typename T>
-__device__ __forceinline__ double cell_rate(const T* q, const MhdCoef<T>& mc) {
-  double rate = 0.0;
-  T Fd[8];
+// max over d of (|v_d| + c_fast,d) / dx_d of a cell, 0 if that is no number.
+// float: kept in float, whose maximum is the same number without conversions
+// and comparisons on the FP64 pipe.  double: the operations of llf_flux2, 73 on
+// that pipe where the IEEE quotients and six IEEE roots make it about 160, and
+// rounded explicitly, so that both of its callers get the same bits.
+__device__ __forceinline__ float cell_rate(const float* q, const MhdCoef<float>& mc) {
+  float rate = 0.0f, Fd[8];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) rate = fmax(rate, double(flux_speed(q, d, mc, Fd) * mc.idx[d]));
+  for (int d = 0; d < 3; ++d) rate = fmaxf(rate, flux_speed(q, d, mc, Fd) * mc.idx[d]);
+  return rate;
+}
+__device__ __forceinline__ double cell_rate(const double* q, const MhdCoef<double>& mc) {
+  const double nir = nrecip1<false>(q[0]);
+  const double* b = q + 5;
+  double nv[3], bb[3];
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    nv[d] = __dmul_rn(q[1 + d], nir);
+    bb[d] = __dmul_rn(b[d], b[d]);
+  }
+  const double B2 = __dadd_rn(__dadd_rn(bb[0], bb[1]), bb[2]);
+  const double nSvB = __fma_rn(q[3], nv[2], __fma_rn(q[2], nv[1], __fma_rn(q[1], nv[0], -B2)));
+  const double pr = __dmul_rn(__dsub_rn(mc.gamma, 1.0), __fma_rn(0.5, nSvB, q[4]));
+  const double na2 = __dmul_rn(__dmul_rn(mc.gamma, pr), nir);
+  const double h = __dmul_rn(-0.5, __fma_rn(B2, nir, na2)), hh = __dmul_rn(h, h);
+  const double n2 = -__dmul_rn(na2, nir);
+  double rate = 0.0;
+#pragma unroll
+  for (int d = 0; d < 3; ++d) {
+    const double disc = __fma_rn(n2, bb[d], hh);
+    const bool below = (unsigned)__double2hiint(disc) - 0x80000000u < 0x7ff00000u;  // finite, < 0
+    const double cf = sqrt1(__dadd_rn(sqrt1(below ? 0.0 : disc), h));
+    rate = fmax(rate, __dmul_rn(__dadd_rn(fabs(nv[d]), cf), mc.idx[d]));  // NaN kept out
+  }
   return rate;
 }
 
@@ -259,7 +287,7 @@ __device__ __forceinline__ void ssp_write(const PatchArgs<T>& a, const StageArgs
 // below, then the face below the first plane).
 //
 // double is bound by the FP64 pipe (one warp instruction per 16 cycles and
-// SM; 86% busy) and reads its stencils from global memory.  float is bound by
+// SM; 92% of its peak) and reads its stencils from global memory.  float is bound by
 // issue and latency (issue 48%, then fixed-latency waits): its planes are
 // staged in shared memory as field pairs by cp.async, five in a ring, so that
 // a stencil value pair is one 64-bit load with a constant offset.  MR + 1 is
@@ -267,8 +295,19 @@ __device__ __forceinline__ void ssp_write(const PatchArgs<T>& a, const StageArgs
 // each where 8 get 255 (float, 9 warps: 1410 us per 128^3 step, 8: 1155).
 // 128^3 SSP-RK3 step with CFL rate, against a kernel that reconstructed each
 // cell once per face and side in tiles of 31 x 11 (float) and 31 x 7 outputs:
-// double 54.5 -> 23.6 ms, float 2.24 -> 0.94 ms.
+// double 54.4 -> 20.3 ms, float 2.22 -> 0.91 ms.
+//
+// A block's work is one chunk of mz planes of one column of tiles or, in
+// double where that is less, an even share of all columns laid end to end,
+// whose boundaries fall between planes: a launch of as many blocks as the GPU
+// holds, all ending together (128^3: 36 columns of 128 planes over 152 SMs,
+// 20.9 -> 20.3 ms).  float keeps to chunks: the loop over the columns of a
+// share costs registers that its planes need (915 -> 965 us).
 constexpr int MX = 32;
+struct MhdWork {
+  int mz;      // planes of a chunk; 0: even shares
+  int nx, ny;  // tiles along x and y
+};
 template <typename T, int MR>
 struct MhdSmem {
   static constexpr bool kStaged = sizeof(T) == 4;
@@ -279,6 +318,7 @@ struct MhdSmem {
   T fy[MR + 1][8][MX];  // y fluxes below rows 0 .. MR
   T exl[8][MR], exr[8][MR], fxr[8][MR];  // x: right edges of cells -1 and 31, flux at 32
   double rate[MR + 1];
+  int work[2], end[2];
   P ring[kStaged ? kSlots : 1][kStaged ? 4 * kCells : 1];  // planes as field pairs
 };
 
@@ -289,21 +329,17 @@ __device__ __forceinline__ void cp_async4(float* dst, const float* src) {
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// One tile's planes k0 .. k1 - 1; the signal rate of the outputs into rate.
 template <typename T, int VAR, int MR>
-__global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
-    mhd_stage_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, int mz) {
+__device__ __forceinline__ void mhd_march(const PatchArgs<T>& a, const StageArgs& s,
+                                          const MhdCoef<T>& mc, MhdSmem<T, MR>& sm, int x0, int y0,
+                                          int k0, int k1, T& rate) {
   using S = MhdSmem<T, MR>;
   using P = typename S::P;
   constexpr int NC = S::kCells, CW = S::kCols;
   constexpr bool ST = S::kStaged;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  S& sm = *reinterpret_cast<S*>(smem_raw);
-  wait_predecessor();
   const int tx = threadIdx.x, ty = threadIdx.y;
   const bool row = ty < MR;
-  const int x0 = blockIdx.x * MX, y0 = blockIdx.y * MR;
-  const int k0 = blockIdx.z * mz;
-  const int k1 = min(k0 + mz, a.n[2]);
   const int g = a.g;
   const int i = x0 + tx, j = y0 + ty;
   const bool out = row && i < a.n[0] && j < a.n[1];
@@ -364,7 +400,6 @@ __global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
       q[2 * f + 1] = P(l[f].y, r[f].y);
     }
   };
-  double rate = 0.0;  // max signal rate of this thread's outputs (fused CFL reduction)
   P erz[4];           // right-edge values along z of the cell below
   T Fzm[8];           // z flux below the current plane
 #pragma unroll
@@ -544,6 +579,57 @@ __global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
     for (int q = 0; q < 4; ++q) sl[q] = sl[q + 1];
     sl[4] = t;
   }
+}
+
+template <typename T, int VAR, int MR>
+__global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
+    mhd_stage_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, MhdWork wk) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  MhdSmem<T, MR>& sm = *reinterpret_cast<MhdSmem<T, MR>*>(smem_raw);
+  wait_predecessor();
+  const bool even = sizeof(T) == 8 && wk.mz == 0, first = threadIdx.x == 0 && threadIdx.y == 0;
+  T rate = 0;  // max signal rate of this thread's outputs (fused CFL reduction)
+  // an even share goes from plane work[1] of column work[0] to before plane
+  // end[1] of column end[0] (in shared memory: the march has no registers to spare)
+  if (even) {
+    if (first) {
+      const int len = 3 * a.n[2] + 2;  // a column in thirds of a plane
+      const long long total = (long long)wk.nx * wk.ny * len;
+      // the first plane that starts at or after boundary b
+      auto cut = [&](unsigned b, int& c, int& k) {
+        const long long at = total * b / gridDim.x;
+        c = (int)(at / len);
+        k = ((int)(at - (long long)c * len) + 2) / 3;
+        if (k >= a.n[2]) {
+          k = 0;
+          ++c;
+        }
+      };
+      cut(blockIdx.x, sm.work[0], sm.work[1]);
+      cut(blockIdx.x + 1, sm.end[0], sm.end[1]);
+    }
+    __syncthreads();
+  }
+#pragma unroll 1
+  while (true) {
+    int bx = blockIdx.x, by = blockIdx.y, k0 = blockIdx.z * wk.mz, k1 = min(k0 + wk.mz, a.n[2]);
+    if (even) {
+      const int col = sm.work[0], last = sm.end[0];
+      k0 = sm.work[1];
+      k1 = col == last ? sm.end[1] : a.n[2];
+      if (col > last || k0 >= k1) break;
+      bx = col % wk.nx;
+      by = col / wk.nx;
+    }
+    mhd_march<T, VAR, MR>(a, s, mc, sm, bx * MX, by * MR, k0, k1, rate);
+    if (!even) break;
+    __syncthreads();  // the next column reuses the shared arrays
+    if (first) {
+      ++sm.work[0];
+      sm.work[1] = 0;
+    }
+    __syncthreads();
+  }
   if (a.rate) block_rate<MR + 1>(rate, sm.rate, a.rate);
 }
 
@@ -645,13 +731,15 @@ __global__ void __launch_bounds__(256) mhd_rate_kernel(const T* __restrict__ u0,
     const int j = (int)((t / nx) % ny);
     const int k = (int)(t / ((long long)nx * ny));
     const T* p = u0 + (long long)(k + g) * sz + (long long)(j + g) * sy + (i + g);
-    T q[8], Fd[8];
+    T q[8];
 #pragma unroll
     for (int f = 0; f < 8; ++f) q[f] = __ldg(p + f * F);
+    if constexpr (sizeof(T) == 8) {
+      best = fmax(best, cell_rate(q, mc));
+    } else {
+      T Fd[8];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-      const double r = double(flux_speed(q, d, mc, Fd)) * double(mc.idx[d]);
-      best = r > best ? r : best;
+      for (int d = 0; d < 3; ++d) best = fmax(best, double(flux_speed(q, d, mc, Fd)) * double(mc.idx[d]));
     }
   }
   // block max, then one atomic per block (non-negative doubles order like their bits)
@@ -688,7 +776,7 @@ static MhdCoef<T> coef(const sf_params& prm, const sf_patch& p) {
 // (3 mz + extra); ties go to the larger mz.  Only chunk lengths whose grid
 // fits gridDim.z (65535) are considered.
 struct MhdPlan {
-  int mz;
+  int mz;  // 0: even shares over `resident` blocks
   long long cost;
 };
 static MhdPlan mhd_planes_per_block(int gx, int gy, int nz, int resident, int extra) {
@@ -735,14 +823,26 @@ struct MhdInstance {
     return cache[dev];
   }
   static MhdPlan plan(const sf_patch& p) {
-    return mhd_planes_per_block((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y, p.n[2],
-                                resident(), ROWS ? 2 : 1);
+    const MhdPlan chunks = mhd_planes_per_block((p.n[0] + out_x - 1) / out_x,
+                                                (p.n[1] + out_y - 1) / out_y, p.n[2], resident(),
+                                                ROWS ? 2 : 1);
+    if (!ROWS || sizeof(T) == 4 || resident() == 0) return chunks;
+    // a share's boundaries are rounded to planes, and it may start inside a column
+    const long long cols = (long long)((p.n[0] + out_x - 1) / out_x) * ((p.n[1] + out_y - 1) / out_y);
+    const long long even = cols * (3LL * p.n[2] + 2) / resident() + 1 + 2 + 2;
+    return even < chunks.cost ? MhdPlan{0, even} : chunks;
   }
   static void launch(const PatchArgs<T>& a, const StageArgs& s, const MhdCoef<T>& mc, const sf_patch& p,
                      int mz, cudaStream_t st) {
     const dim3 block(MX, threads_y, 1);
-    const dim3 grid((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y, (p.n[2] + mz - 1) / mz);
-    launch_after(kernel(), grid, block, smem, st, a, s, mc, mz);
+    const dim3 grid((p.n[0] + out_x - 1) / out_x, (p.n[1] + out_y - 1) / out_y,
+                    mz ? (p.n[2] + mz - 1) / mz : 1);
+    if constexpr (ROWS == 0) {
+      launch_after(kernel(), grid, block, smem, st, a, s, mc, mz);
+    } else {
+      const MhdWork wk = {mz, (int)grid.x, (int)grid.y};
+      launch_after(kernel(), mz ? grid : dim3(resident()), block, smem, st, a, s, mc, wk);
+    }
   }
 };
 

@@ -11,7 +11,7 @@
 // the nonlinear weights are linear weight x P_k with the same P_k for both
 // edges.  The edge value is the cell's value plus a correction, so a uniform
 // state is reproduced exactly and the correction's rounding is relative to
-// the correction.  47 operations give both edges (double) (App. B evaluated per face
+// the correction.  41 operations give both edges (double) (App. B evaluated per face
 // and per side takes about 124 for the same two values).
 #pragma once
 
@@ -244,21 +244,21 @@ __device__ __forceinline__ void weno_edges(const P* w, T eps, const MhdCoef<T>& 
     el = fma2(fma2(two, q1, q0), il, w[2]);
     return;
   }
-  // beta_k = 4/3 a_k^2 + a product of differences (13/12 a^2 + 1/4 b^2 of App. B
-  // with b expressed by a and the differences)
+  // beta_k = a_k (4/3 a_k -+ d) + d^2 (13/12 a^2 + 1/4 b^2 of App. B with b
+  // expressed by a and a difference), d^2 + eps shared
   const P d0 = sub2(w[1], w[0]), d3 = sub2(w[4], w[3]);
   const P a0 = sub2(d3, d2), a1 = sub2(d2, d1), a2 = sub2(d1, d0);
   const P c43(T(4.0 / 3.0)), ep(eps);
-  const P e0 = fma2(d2, sub2(d2, a0), fma2(mul2(c43, a0), a0, ep));
-  const P e1 = fma2(d1, d2, fma2(mul2(c43, a1), a1, ep));
-  const P e2 = fma2(d1, add2(d1, a2), fma2(mul2(c43, a2), a2, ep));
+  const P g1 = fma2(d1, d1, ep), g2 = fma2(d2, d2, ep);
+  const P e0 = fma2(a0, fma2(c43, a0, neg2(d2)), g2);
+  const P e1 = fma2(a1, fma2(c43, a1, d1), g1);
+  const P e2 = fma2(a2, fma2(c43, a2, d1), g1);
   P p0, p1, p2;
   weno_weights<VAR>(e0, e1, e2, mc, p0, p1, p2);
   // right edge: weights 3 p0, 6 p1, p2; left edge: p0, 6 p1, 3 p2
   const P two(T(2)), three(T(3)), mt(T(-2.0 / 3.0));
-  const P s6 = mul2(P(T(6)), p1);
-  const P sr = add2(fma2(three, p0, s6), p2), sl = add2(fma2(three, p2, s6), p0);
   const P ur = fma2(two, p1, p2), ul = fma2(two, p1, p0);
+  const P sr = fma2(three, ul, p2), sl = fma2(three, ur, p0);
   const P q0 = mul2(p0, a0), q2 = mul2(p2, a2);
   const P nr = fma2(mt, q2, fma2(ur, a1, q0));
   const P nl = fma2(mt, q0, fma2(ul, a1, q2));
@@ -280,27 +280,36 @@ __device__ __forceinline__ void llf_flux2(const P* q, T gamma, T* F) {
   const P* b = q + 5;
   const P bd2 = mul2(b[D], b[D]);
   const P B2 = fma2(b[B], b[B], fma2(b[A], b[A], bd2));
-  const P nSv = fma2(q[3], nv[2], fma2(q[2], nv[1], mul2(q[1], nv[0])));
-  const P pr = mul2(P(gamma - T(1)), fma2(P(T(0.5)), sub2(nSv, B2), q[4]));
+  const P nSvB = fma2(q[3], nv[2], fma2(q[2], nv[1], fma2(q[1], nv[0], neg2(B2))));
+  const P pr = mul2(P(gamma - T(1)), fma2(P(T(0.5)), nSvB, q[4]));
   const P pt = fma2(P(T(0.5)), B2, pr);
   const P nvB = fma2(nv[2], b[2], fma2(nv[1], b[1], mul2(nv[0], b[0])));
   const P nb = neg2(b[D]);
   const P Sd = q[1 + D];
   // signal speed |v_d| + c_fast
   const P na2 = mul2(mul2(P(gamma), pr), nir);
-  const P ns = fma2(B2, nir, na2);
-  const P disc = fma2(mul2(P(T(-4)), na2), mul2(bd2, nir), mul2(ns, ns));
-  const P cf = sqrt2(mul2(P(T(0.5)), sub2(sqrt2(pos2(disc)), ns)));
+  const P h = mul2(P(T(-0.5)), fma2(B2, nir, na2));
+  const P disc = fma2(neg2(na2), mul2(bd2, nir), mul2(h, h));
+  const P cf = sqrt2(add2(sqrt2(pos2(disc)), h));
   const T S = larger(fabs(nv[D].x) + cf.x, fabs(nv[D].y) + cf.y);
   auto out = [&](int f, P nf) { F[f] = fma(-S, q[f].y - q[f].x, -nf.x - nf.y); };
   F[0] = fma(-S, q[0].y - q[0].x, Sd.x + Sd.y);
   out(1 + D, sub2(fma2(Sd, nv[D], bd2), pt));
-  out(1 + A, fma2(b[D], b[A], mul2(Sd, nv[A])));
-  out(1 + B, fma2(b[D], b[B], mul2(Sd, nv[B])));
-  out(4, fma2(nb, nvB, mul2(add2(q[4], pt), nv[D])));
+  // u v + w z of both states: in double one chain over the states
+  auto out4 = [&](int f, P u, P v, P w, P z) {
+    if constexpr (sizeof(T) == 8) {
+      const T t = fma(w.y, z.y, fma(w.x, z.x, fma(u.y, v.y, u.x * v.x)));
+      F[f] = fma(-S, q[f].y - q[f].x, -t);
+    } else {
+      out(f, fma2(w, z, mul2(u, v)));
+    }
+  };
+  out4(1 + A, Sd, nv[A], b[D], b[A]);
+  out4(1 + B, Sd, nv[B], b[D], b[B]);
+  out4(4, add2(q[4], pt), nv[D], nb, nvB);
   F[5 + D] = fma(-S, b[D].y - b[D].x, T(0));
-  out(5 + A, fma2(nb, nv[A], mul2(nv[D], b[A])));
-  out(5 + B, fma2(nb, nv[B], mul2(nv[D], b[B])));
+  out4(5 + A, nv[D], b[A], nb, nv[A]);
+  out4(5 + B, nv[D], b[B], nb, nv[B]);
 }
 
 }  // namespace sf

@@ -48,6 +48,7 @@ def _check(n, precision, prm, floor, U0, dx):
 
 SIZES = [(31, 14, 4), (32, 15, 4), (33, 16, 4), (64, 30, 3), (65, 31, 5), (3, 8, 3), (33, 21, 40),
          (33, 7, 160)]
+EVEN = [(129, 50, 50), (352, 210, 3)]
 
 
 @pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
@@ -55,6 +56,14 @@ SIZES = [(31, 14, 4), (32, 15, 4), (33, 16, 4), (64, 30, 3), (65, 31, 5), (3, 8,
 def test_tile_edges(n, precision):
     U0, dx = inputs.mhd_blast(n, seed=sum(n), radius=0.3)
     _check(n, precision, capi.params(rk=capi.SF_SSPRK3), [1e-3] * 8, U0, dx)
+
+
+# sizes at which double blocks take even shares of all columns on 152 SMs:
+# shares that start inside a column, and shares of more than one column
+@pytest.mark.parametrize("n", EVEN)
+def test_even_shares(n):
+    U0, dx = inputs.mhd_blast(n, seed=sum(n), radius=0.3)
+    _check(n, capi.SF_FP64, capi.params(rk=capi.SF_SSPRK3), [1e-3] * 8, U0, dx)
 
 
 @pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
