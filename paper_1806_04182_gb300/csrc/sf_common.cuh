@@ -104,7 +104,11 @@ __device__ __forceinline__ T ko_all(const T* __restrict__ p, long long sy, long 
   return kc[0] * delta6(p, 1, c0) + kc[1] * delta6(p, sy, c0) + kc[2] * delta6(p, sz, c0);
 }
 
-__device__ __forceinline__ bool finite_(double v) { return isfinite(v); }
+// (by its exponent bits: a double comparison takes the FP64 pipe, 1% of an FP64
+// CCZ4 stage)
+__device__ __forceinline__ bool finite_(double v) {
+  return ((unsigned)__double2hiint(v) & 0x7ff00000u) != 0x7ff00000u;
+}
 __device__ __forceinline__ bool finite_(float v) { return isfinite(v); }
 
 // ------------------------------------------------------------ stage write

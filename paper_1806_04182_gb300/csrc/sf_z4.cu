@@ -9,9 +9,16 @@
 
 namespace sf {
 
-// 128 threads and at least 3 CTAs per SM for the float kernels (<= 168
-// registers): on the 96^3 benchmark patch this measured faster than 2 CTAs
-// (255 registers) and than 4+ CTAs (128 registers or fewer, with spills).
+// 128 threads and at least MINB CTAs per SM.  float: 3 (<= 168 registers): on
+// the 96^3 benchmark patch this measured faster than 2 CTAs (255 registers)
+// and than 4+ CTAs (128 registers or fewer, with spills).  double is bound by
+// the FP64 pipe (2435 operations a point; 87% busy at 2 CTAs): 3 CTAs spill
+// but leave the pipe less idle between loads and writes, where the patch gives
+// more than 2 CTAs to every SM (96^3 step 15.99 -> 15.90 ms, 61 x 47 x 53 3.28
+// -> 3.10 ms, with one-sided advection 4.38 -> 4.04 ms; below that line the
+// spills only lengthen the one round: 20^3 395 against 406 us, 32^3 730 against
+// 735 us).  In z4_rhs's order of operations (2820 a point) the 96^3 step took
+// 18.65 ms.
 //
 // The right-hand sides of the 25 fields are parked in shared memory as
 // z4_cell produces them, and the RK stage combination (which reads U^n, the
@@ -19,8 +26,8 @@ namespace sf {
 // rolled loop over the fields.  Inlined after every field, the combination
 // put 25 copies of its code and 25 dependent DRAM reads into the middle of the
 // computation; the deferred form measured 7-10% faster on the 96^3 patch.
-template <typename T, typename H, int SY, int SZ, bool LOP>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2)
+template <typename T, typename H, int SY, int SZ, bool LOP, int MINB>
+__global__ void __launch_bounds__(128, MINB)
     z4_stage_kernel(PatchArgs<T> a, StageArgs s, Z4Coef<T> zc) {
   __shared__ T rbuf[25 * 128];
   wait_predecessor();
@@ -39,19 +46,40 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2)
   write_fields<T, 25>(a, s, im, c, i, j, k, rbuf + tid, 128);
 }
 
+static int sm_count() {
+  static int cache[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cache[dev] && cudaDeviceGetAttribute(&cache[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    cache[dev] = 0;
+  return cache[dev];
+}
+
+template <typename T, typename H, int MINB>
+static void launch_kernel(const PatchArgs<T>& a, const StageArgs& s, const sf_params& prm, const sf_patch& p,
+                          dim3 grid, cudaStream_t st) {
+  const Z4Coef<T> zc = z4_coef<T>(prm);
+  const dim3 block(32, 4, 1);
+  if (prm.lopsided)
+    launch_after(z4_stage_kernel<T, H, 0, 0, true, MINB>, grid, block, 0, st, a, s, zc);
+  else if (p.sy == 102 && p.sz == 102 * 102)
+    launch_after(z4_stage_kernel<T, H, 102, 102 * 102, false, MINB>, grid, block, 0, st, a, s, zc);
+  else
+    launch_after(z4_stage_kernel<T, H, 0, 0, false, MINB>, grid, block, 0, st, a, s, zc);
+}
+
 template <typename T, typename H>
 static sf_status launch(const sf_params& prm, const sf_patch& p, const StageArgs& s, int stage,
                         void* rhs_out, cudaStream_t st) {
-  PatchArgs<T> a = make_args<T>(prm, p, stage, 25, rhs_out);
-  const Z4Coef<T> zc = z4_coef<T>(prm);
-  dim3 block(32, 4, 1);
-  dim3 grid((p.n[0] + 31) / 32, (p.n[1] + 3) / 4, p.n[2]);
-  if (prm.lopsided)
-    launch_after(z4_stage_kernel<T, H, 0, 0, true>, grid, block, 0, st, a, s, zc);
-  else if (p.sy == 102 && p.sz == 102 * 102)
-    launch_after(z4_stage_kernel<T, H, 102, 102 * 102, false>, grid, block, 0, st, a, s, zc);
-  else
-    launch_after(z4_stage_kernel<T, H, 0, 0, false>, grid, block, 0, st, a, s, zc);
+  const PatchArgs<T> a = make_args<T>(prm, p, stage, 25, rhs_out);
+  const dim3 grid((p.n[0] + 31) / 32, (p.n[1] + 3) / 4, p.n[2]);
+  if constexpr (sizeof(T) == 8) {
+    if ((long long)grid.x * grid.y * grid.z <= 2LL * sm_count()) {
+      launch_kernel<T, H, 2>(a, s, prm, p, grid, st);
+      return after_launch("z4_stage_kernel");
+    }
+  }
+  launch_kernel<T, H, 3>(a, s, prm, p, grid, st);
   return after_launch("z4_stage_kernel");
 }
 

@@ -664,12 +664,20 @@ __device__ __forceinline__ void z4_rhs(const ZC& zc, Sten& sten, V (&be)[3], Out
   sten.finish();
 }
 
+}  // namespace sf
+#include "sf_z4_fp64.cuh"
+namespace sf {
+
 template <typename T, typename H, bool LOP, typename Src, typename Out>
 __device__ __forceinline__ void z4_cell(const PatchArgs<T>& a, const Z4Coef<T>& zc, Src& src,
                                         Out&& out) {
-  T be[3];
-  Z4Sten<T, LOP, Src> sten{a, src, be};
-  z4_rhs<T, H, LOP>(zc, sten, be, out);
+  if constexpr (sizeof(T) == 8) {
+    z4_rhs64<LOP>(a, zc, src, out);
+  } else {
+    T be[3];
+    Z4Sten<T, LOP, Src> sten{a, src, be};
+    z4_rhs<T, H, LOP>(zc, sten, be, out);
+  }
 }
 
 }  // namespace sf
