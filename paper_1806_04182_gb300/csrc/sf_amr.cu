@@ -116,7 +116,7 @@ __device__ __forceinline__ int floordiv(int a, int b) { return a >= 0 ? a / b : 
 template <typename T>
 struct Combo {
   const T* s[5];
-  double c[4];
+  T c[4];  // (converted in every thread they took the FP64 pipe)
 };
 
 // Formed in the arrays' own precision: float arrays hold values to float
@@ -127,7 +127,7 @@ __device__ __forceinline__ T node_value(const Combo<T>& cb, long long o) {
   if (NS > 0) {
     const T u = v;
 #pragma unroll
-    for (int m = 1; m <= NS; ++m) v += T(cb.c[m - 1]) * (__ldg(cb.s[m] + o) - u);
+    for (int m = 1; m <= NS; ++m) v += cb.c[m - 1] * (__ldg(cb.s[m] + o) - u);
   }
   return v;
 }
@@ -677,7 +677,7 @@ static sf_status prolong_launch(const sf_patch* coarse, const void* const* array
     } else {
       Combo<float> cb;
       for (int m = 0; m < 5; ++m) cb.s[m] = m <= NS ? (const float*)arrays[m] : nullptr;
-      for (int m = 0; m < 4; ++m) cb.c[m] = (c && m < NS) ? c[m] : 0.0;
+      for (int m = 0; m < 4; ++m) cb.c[m] = (c && m < NS) ? (float)c[m] : 0.0f;
       static std::once_flag once;
       std::call_once(once, [] {
         cudaFuncSetAttribute(prolong_kernel<float, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
