@@ -772,16 +772,18 @@ static MhdCoef<T> coef(const sf_params& prm, const sf_patch& p) {
 // Planes per block along z: a block evaluates mz planes and the passes before
 // its first one, about (3 mz + extra) / 3 planes' work, and a launch of B
 // blocks takes ceil(B / resident) rounds of the resident blocks (blocks per
-// SM x SMs), so mz in [1, 32] minimises the cost ceil(B(mz) / resident)
-// (3 mz + extra); ties go to the larger mz.  Only chunk lengths whose grid
-// fits gridDim.z (65535) are considered.
+// SM x SMs), so mz in [lo, hi] minimises the cost ceil(B(mz) / resident)
+// (3 mz + extra); ties go to the larger mz.  The split kernel, which reads its
+// stencils from global memory, keeps to 4 .. 16 planes (99 x 48 x 88 float in 1
+// .. 32: 1036 instead of 1021 us).  Only chunk lengths whose grid fits gridDim.z
+// (65535) are considered.
 struct MhdPlan {
   int mz;  // 0: even shares over `resident` blocks
   long long cost;
 };
-static MhdPlan mhd_planes_per_block(int gx, int gy, int nz, int resident, int extra) {
-  MhdPlan best = {32, -1};
-  for (int mz = 32; mz >= 1; --mz) {
+static MhdPlan mhd_planes_per_block(int gx, int gy, int nz, int resident, int extra, int lo, int hi) {
+  MhdPlan best = {hi, -1};
+  for (int mz = hi; mz >= lo; --mz) {
     if ((nz + mz - 1) / mz > 65535) break;
     const long long blocks = (long long)gx * gy * ((nz + mz - 1) / mz);
     const long long rounds = resident > 0 ? (blocks + resident - 1) / resident : blocks;
@@ -825,7 +827,7 @@ struct MhdInstance {
   static MhdPlan plan(const sf_patch& p) {
     const MhdPlan chunks = mhd_planes_per_block((p.n[0] + out_x - 1) / out_x,
                                                 (p.n[1] + out_y - 1) / out_y, p.n[2], resident(),
-                                                ROWS ? 2 : 1);
+                                                ROWS ? 2 : 1, ROWS ? 1 : 4, ROWS ? 32 : 16);
     if (!ROWS || sizeof(T) == 4 || resident() == 0) return chunks;
     // a share's boundaries are rounded to planes, and it may start inside a column
     const long long cols = (long long)((p.n[0] + out_x - 1) / out_x) * ((p.n[1] + out_y - 1) / out_y);

@@ -4,6 +4,8 @@
 // TMA-staged kernels (sf_z4_tma.cu).  Layouts with the
 // strides of a dense 96^3 patch with 3 ghosts get a kernel with compile-time
 // strides; every other layout, and one-sided advection, uses runtime strides.
+#include <algorithm>
+
 #include "sf_internal.cuh"
 #include "sf_z4.cuh"
 
@@ -13,12 +15,13 @@ namespace sf {
 // the 96^3 benchmark patch this measured faster than 2 CTAs (255 registers)
 // and than 4+ CTAs (128 registers or fewer, with spills).  double is bound by
 // the FP64 pipe (2435 operations a point; 87% busy at 2 CTAs): 3 CTAs spill
-// but leave the pipe less idle between loads and writes, where the patch gives
-// more than 2 CTAs to every SM (96^3 step 15.99 -> 15.90 ms, 61 x 47 x 53 3.28
-// -> 3.10 ms, with one-sided advection 4.38 -> 4.04 ms; below that line the
-// spills only lengthen the one round: 20^3 395 against 406 us, 32^3 730 against
-// 735 us).  In z4_rhs's order of operations (2820 a point) the 96^3 step took
-// 18.65 ms.
+// but leave the pipe less idle between loads and writes (96^3 step 15.99 ->
+// 15.90 ms, 61 x 47 x 53 3.28 -> 3.10 ms, with one-sided advection 4.38 -> 4.04
+// ms), except where an SM's share of the patch is 1, 2 or 4 CTAs: up to 2 the
+// spills only lengthen the one round (20^3 395 against 406 us, 32^3 730 against
+// 735 us), and 3 + 1 leaves the last CTA alone where 2 + 2 does not (37 x 55 x
+// 19 one-sided SHARE4).  In z4_rhs's order of operations (2820 a point) the
+// 96^3 step took 18.65 ms.
 //
 // The right-hand sides of the 25 fields are parked in shared memory as
 // z4_cell produces them, and the RK stage combination (which reads U^n, the
@@ -74,7 +77,9 @@ static sf_status launch(const sf_params& prm, const sf_patch& p, const StageArgs
   const PatchArgs<T> a = make_args<T>(prm, p, stage, 25, rhs_out);
   const dim3 grid((p.n[0] + 31) / 32, (p.n[1] + 3) / 4, p.n[2]);
   if constexpr (sizeof(T) == 8) {
-    if ((long long)grid.x * grid.y * grid.z <= 2LL * sm_count()) {
+    const long long sms = std::max(1, sm_count());
+    const long long share = ((long long)grid.x * grid.y * grid.z + sms - 1) / sms;
+    if (share <= 2 || share == 4) {
       launch_kernel<T, H, 2>(a, s, prm, p, grid, st);
       return after_launch("z4_stage_kernel");
     }
