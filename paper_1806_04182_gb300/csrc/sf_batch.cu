@@ -132,7 +132,7 @@ struct sf_batch {
   void* d_pcoefs = nullptr;  // its stencil weights, one block per patch
   TmaTile* d_ptiles = nullptr;  // its tiles, those of shape 0, then of shape 1
   int npair = 0;                // two-point tiles
-  int nwide = 0;                // of which the first nwide are of shape 0
+  int pair_ends[3] = {0, 0, 0};  // where those of each shape (kPairShapes) end
   void* d_maps = nullptr; // tensor maps, 3 per patch (u_n, u_stage, u_next roles)
   TmaTile* d_tiles = nullptr;   // 32 x 12 tiles, then 16 x 24 tiles
   int ntiles = 0;               // all TMA tiles
@@ -222,27 +222,35 @@ sf_status build_items(sf_batch* b, int only_class) {
 // not a multiple.
 sf_status build_pair(sf_batch* b) {
   b->pair.assign(b->npatch, 0);
-  b->npair = b->nwide = 0;
+  b->npair = 0;
   if (b->precision != SF_FP32_BULK_DW) return SF_OK;
   const size_t cb = z4_pair_coef_bytes();
   std::vector<unsigned char> maps((size_t)6 * b->npatch * kTmaMapBytes, 0), coefs(cb * b->npatch, 0);
-  std::vector<TmaTile> lists[2];
+  std::vector<TmaTile> lists[3];
+  int only = -1;  // the one shape that all patches take, 3 if they differ
+  for (const sf_patch& p : b->patches) {
+    if (!z4_pair_batch_eligible(b->prm, p)) continue;
+    const int w = z4_pair_shape(p, 0);
+    only = only < 0 || only == w ? w : 3;
+  }
   for (int q = 0; q < b->npatch; ++q) {
     const sf_patch& p = b->patches[q];
     if (!z4_pair_batch_eligible(b->prm, p)) continue;
     b->pair[q] = 1;
+    const int w = only < 3 ? only : z4_pair_shape(p, 1);
     sf_status e = encode_z4_pair_batch(maps.data() + (size_t)6 * q * kTmaMapBytes, coefs.data() + cb * q,
-                                       b->prm, p);
+                                       b->prm, p, w);
     if (e) return e;
-    const int w = z4_pair_shape(p);
     const int* t = kPairShapes[w];
     for (int z = 0; z < p.n[2]; z += t[2])
       for (int y = 0; y < p.n[1]; y += t[1])
         for (int x = 0; x < p.n[0]; x += t[0]) lists[w].push_back(TmaTile{q, x, y, z});
   }
   std::vector<TmaTile>& tiles = lists[0];
-  b->nwide = (int)tiles.size();
-  tiles.insert(tiles.end(), lists[1].begin(), lists[1].end());
+  for (int w = 0; w < 3; ++w) {
+    if (w) tiles.insert(tiles.end(), lists[w].begin(), lists[w].end());
+    b->pair_ends[w] = (int)tiles.size();
+  }
   b->npair = (int)tiles.size();
   if (tiles.empty()) return SF_OK;
   if (cudaMalloc(&b->d_pmaps, maps.size()) != cudaSuccess ||
@@ -331,8 +339,10 @@ sf_status launch_stage(sf_batch* b, int stage, cudaStream_t st, unsigned int* st
     const PatchArgs<float>* fargs =
         static_cast<const PatchArgs<float>*>(b->d_args) + (size_t)stage * b->npatch;
     const StageArgs sa = batch_stage_args(b, stage, status);
-    sf_status e = launch_z4_pair_batch(b->prm, b->d_pmaps, role[stage], fargs, b->d_pcoefs,
-                                       b->d_ptiles, b->npair, b->nwide, sa, st);
+    sf_status e = SF_OK;
+    if (b->npair > 0)
+      e = launch_z4_pair_batch(b->prm, b->d_pmaps, role[stage], fargs, b->d_pcoefs, b->d_ptiles,
+                               b->pair_ends, sa, st);
     const int n32 = b->ntiles - b->ntiles16;
     if (!e)
       e = launch_z4_tma_batch(b->prm, b->precision, b->d_maps, role[stage], fargs, b->d_tiles, n32,

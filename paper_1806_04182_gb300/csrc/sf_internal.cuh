@@ -43,20 +43,19 @@ constexpr int kTmaTileX = 32, kTmaTileY = 12;      // the wide tile
 constexpr int kTmaTileX16 = 16, kTmaTileY16 = 24;  // the narrow tile
 constexpr size_t kTmaMapBytes = 128;  // sizeof(CUtensorMap)
 bool z4_tma_batch_eligible(const sf_params& prm, const sf_patch& p);
-// Two-point tiles of many patches (sf_z4_pair_any.cu) of two shapes, for float
+// Two-point tiles of many patches (sf_z4_pair_batch.cu) of three shapes, for float
 // CCZ4 batch patches with double-word islands on the one-float row offset
 // layout: six tensor maps per patch (RK chunks of u_n, acc, kahan; stencil
 // boxes of the u_n, u_stage, u_next roles, for the patch's shape) and the
 // patch's stencil weights (z4_pair_coef_bytes each) in device memory.
-constexpr int kPairShapes[2][3] = {{32, 8, 2}, {16, 8, 4}};
-int z4_pair_shape(const sf_patch& p);  // the shape that covers p with fewer tiles
+constexpr int kPairShapes[3][3] = {{32, 16, 1}, {32, 8, 2}, {16, 8, 4}};
+int z4_pair_shape(const sf_patch& p, int first);  // the shape from `first` on that covers p in the least time
 bool z4_pair_batch_eligible(const sf_params& prm, const sf_patch& p);
 size_t z4_pair_coef_bytes();
-sf_status encode_z4_pair_batch(void* maps6, void* coef, const sf_params& prm, const sf_patch& p);
+sf_status encode_z4_pair_batch(void* maps6, void* coef, const sf_params& prm, const sf_patch& p, int w);
 sf_status launch_z4_pair_batch(const sf_params& prm, const void* d_maps, int role,
                                const PatchArgs<float>* d_args, const void* d_coefs,
-                               const TmaTile* d_tiles, int ntiles, int nwide, const StageArgs& s,
-                               cudaStream_t st);
+                               const TmaTile* d_tiles, const int* ends, const StageArgs& s, cudaStream_t st);
 sf_status encode_z4_tma_map(void* map, const sf_patch& p, const void* base, int xp);
 sf_status launch_z4_tma_batch(const sf_params& prm, int precision, const void* d_maps, int role,
                               const PatchArgs<float>* d_args, const TmaTile* d_tiles, int ntiles,

@@ -20,7 +20,7 @@ namespace sf {
 // ms), except where an SM's share of the patch is 1, 2 or 4 CTAs: up to 2 the
 // spills only lengthen the one round (20^3 395 against 406 us, 32^3 730 against
 // 735 us), and 3 + 1 leaves the last CTA alone where 2 + 2 does not (37 x 55 x
-// 19 one-sided SHARE4).  In z4_rhs's order of operations (2820 a point) the
+// 19 one-sided 2.19 against 1.84 ms).  In z4_rhs's order of operations (2820 a point) the
 // 96^3 step took 18.65 ms.
 //
 // The right-hand sides of the 25 fields are parked in shared memory as

@@ -94,6 +94,9 @@ struct PairShape {
 // and from 7310 to 6960 warp instructions per warp (96^3 step 985 -> 970 us,
 // sub-cycled 64^3 pair 1667 -> 1555 us).
 using PairFlat = PairShape<32, 16, 1, 7, 12>;
+// 8 slots for the tiles of several planes (9, 7 and 5: 3%, 1% and 4% slower on eight 48^3 patches)
+using PairWide = PairShape<32, 8, 2, 8, 9>;
+using PairDeep = PairShape<16, 8, 4, 8, 9>;
 
 // Order in which z4_rhs opens the fields' stencils.  Without the
 // Gamma-driver (shift frozen) the last three are not used.

@@ -1,29 +1,31 @@
 // The two-point CCZ4 tile (sf_z4_pair.cuh) for patches of any size on the
 // one-float row offset layout: runtime strides, tiles that overhang the patch
-// with masked stores, one patch per launch or the tiles of many patches.
+// with masked stores, one patch per launch (sf_z4_pair_batch.cu: the tiles of
+// many patches).
 //
-// Two tile shapes of 512 points, 32 x 8 x 2 and 16 x 8 x 4; a patch takes the one
-// that covers it with fewer tiles (kPairShapes; the wide one on a tie).  Lanes
-// outside the patch idle: with 32 x 16 x 1 tiles alone, 36% of them on patches
-// of 16 to 64 points a side and 25% on 48^3, with the two shapes 23% and none
-// (96 mixed patches 11.6 -> 10.0 ms per RK4 step, eight 48^3 patches with halo
-// exchange 1.59 -> 1.36 ms; a multi-plane tile by itself costs some 15% more
-// than a flat one, so the padded 96^3-class layout keeps those).
+// Three tile shapes of 512 points, 32 x 16 x 1, 32 x 8 x 2 and 16 x 8 x 4
+// (kPairShapes).  Lanes outside the patch idle: with 32 x 16 x 1 tiles alone,
+// 36% of them on patches of 16 to 64 points a side and 25% on 48^3 (96 mixed
+// patches 11.6 ms per RK4 step, eight 48^3 patches with halo exchange 1.59; with
+// the other two alone 10.0 and 1.36).  A tile of two or four planes takes some
+// 15% or 20% longer than a flat one (96^3, which all three cover exactly), so a
+// patch takes the shape with the least tiles x time (four 36 x 41 x 17 patches:
+// 400 us a step with the other two, 336 with all three).
 #include "sf_z4_pair.cuh"
 
 namespace sf {
 
-// 8 slots each (9, 7 and 5: 3%, 1% and 4% slower on eight 48^3 patches)
-using PairWide = PairShape<32, 8, 2, 8, 9>;
-using PairDeep = PairShape<16, 8, 4, 8, 9>;
-
-int z4_pair_shape(const sf_patch& p) {
+int z4_pair_shape(const sf_patch& p, int first) {
   auto tiles = [&](const int* t) {
     long long n = 1;
     for (int d = 0; d < 3; ++d) n *= (p.n[d] + t[d] - 1) / t[d];
     return n;
   };
-  return tiles(kPairShapes[1]) < tiles(kPairShapes[0]) ? 1 : 0;
+  constexpr int time[3] = {20, 23, 24};
+  int best = first;
+  for (int w = first + 1; w < 3; ++w)
+    if (tiles(kPairShapes[w]) * time[w] < tiles(kPairShapes[best]) * time[best]) best = w;
+  return best;
 }
 
 // One CTA per tile of one patch (the RK4 Kahan forms).
@@ -37,41 +39,6 @@ __global__ void __launch_bounds__(C::kThreads, 1)
   const int z = (int)((blockIdx.z + 3 * gridDim.z - 3) % gridDim.z);
   pair_tile<DW2, C, FORM, true>(&map, rk.m, a, s, zc, &pc, blockIdx.x * C::BX, blockIdx.y * C::BY,
                                 z * C::BZ, smem);
-}
-
-// The same over the tiles of many patches (the float CCZ4 patches of a batch
-// on the two-point layout): one CTA per tile, the first n0 of the wide shape,
-// the rest of the deep one; the tile's patch from `tl`, its stage arguments
-// and stencil weights copied into shared memory, its tensor maps from `maps`
-// (six per patch: RK chunks of U^n, accumulator and Kahan term, then the
-// stencil boxes of the u_n, u_stage and u_next buffer roles; `role` picks the
-// stage input).
-template <int FORM>
-__global__ void __launch_bounds__(32 * kPairWarps, 1)
-    z4_pair_batch_kernel(const CUtensorMap* __restrict__ maps, int role,
-                         const PatchArgs<float>* __restrict__ args, const PairCoef* __restrict__ coefs,
-                         const TmaTile* __restrict__ tl, int n0, StageArgs s, Z4Coef<float> zc) {
-  extern __shared__ __align__(128) unsigned char smem[];
-  __shared__ PatchArgs<float> pa;
-  __shared__ PairCoef pcs;
-  wait_predecessor();
-  const TmaTile w = tl[blockIdx.x];
-  {
-    static_assert(sizeof(PatchArgs<float>) % 4 == 0 && sizeof(PairCoef) % 4 == 0, "word copy");
-    const int tid = threadIdx.y * 32 + threadIdx.x;
-    const int* from = reinterpret_cast<const int*>(args + w.patch);
-    int* to = reinterpret_cast<int*>(&pa);
-    for (int q = tid; q < (int)(sizeof(PatchArgs<float>) / 4); q += 32 * kPairWarps) to[q] = from[q];
-    from = reinterpret_cast<const int*>(coefs + w.patch);
-    to = reinterpret_cast<int*>(&pcs);
-    for (int q = tid; q < (int)(sizeof(PairCoef) / 4); q += 32 * kPairWarps) to[q] = from[q];
-  }
-  // (pair_tile's first barrier orders these copies before their reads)
-  const CUtensorMap* pm = maps + 6 * (size_t)w.patch;
-  if ((int)blockIdx.x < n0)
-    pair_tile<DW2, PairWide, FORM, true>(pm + 3 + role, pm, pa, s, zc, &pcs, w.x0, w.y0, w.z0, smem);
-  else
-    pair_tile<DW2, PairDeep, FORM, true>(pm + 3 + role, pm, pa, s, zc, &pcs, w.x0, w.y0, w.z0, smem);
 }
 
 namespace {
@@ -107,17 +74,6 @@ sf_status launch_any(const sf_params& prm, const sf_patch& p, const StageArgs& s
   return after_launch("z4_pair_any_kernel");
 }
 
-template <typename C>
-sf_status encode_batch(void* maps6, const sf_patch& p) {
-  const void* arr[6] = {p.u_n, p.acc, p.kahan, p.u_n, p.u_stage, p.u_next};
-  for (int q = 0; q < 6; ++q) {
-    CUtensorMap m;
-    if (sf_status e = encode_pair_map<C>(&m, p, arr[q], q < 3)) return e;
-    memcpy(static_cast<char*>(maps6) + q * sizeof(CUtensorMap), &m, sizeof(m));
-  }
-  return SF_OK;
-}
-
 }  // namespace
 
 // Any size on the one-float row offset layout: double-word islands, the RK4
@@ -131,8 +87,11 @@ bool z4_pair_any_eligible(const sf_params& prm, const sf_patch& p, const StageAr
 
 sf_status launch_z4_pair_any(const sf_params& prm, const sf_patch& p, const StageArgs& s, int stage,
                              cudaStream_t st) {
-  if (z4_pair_shape(p)) return launch_any<PairDeep>(prm, p, s, stage, st);
-  return launch_any<PairWide>(prm, p, s, stage, st);
+  switch (z4_pair_shape(p, 0)) {
+    case 0: return launch_any<PairFlat>(prm, p, s, stage, st);
+    case 1: return launch_any<PairWide>(prm, p, s, stage, st);
+    default: return launch_any<PairDeep>(prm, p, s, stage, st);
+  }
 }
 
 // Batch form: float CCZ4 with double-word islands, centred advection, 3
@@ -146,50 +105,6 @@ bool z4_pair_batch_eligible(const sf_params& prm, const sf_patch& p) {
                         (const void*)p.acc, (const void*)p.kahan})
     if (!offset_aligned(q)) return false;
   return true;
-}
-
-size_t z4_pair_coef_bytes() { return sizeof(PairCoef); }
-
-// The six tensor maps of a batch patch (RK chunks of u_n, acc, kahan; stencil
-// boxes of u_n, u_stage, u_next) for its tile shape, and its stencil weights.
-sf_status encode_z4_pair_batch(void* maps6, void* coef, const sf_params& prm, const sf_patch& p) {
-  if (sf_status e = z4_pair_shape(p) ? encode_batch<PairDeep>(maps6, p) : encode_batch<PairWide>(maps6, p))
-    return e;
-  const PairCoef pc = pair_coef(prm, p);
-  memcpy(coef, &pc, sizeof(pc));
-  return SF_OK;
-}
-
-sf_status launch_z4_pair_batch(const sf_params& prm, const void* d_maps, int role,
-                               const PatchArgs<float>* d_args, const void* d_coefs,
-                               const TmaTile* d_tiles, int ntiles, int nwide, const StageArgs& s,
-                               cudaStream_t st) {
-  if (ntiles <= 0) return SF_OK;
-  constexpr int smem =
-      PairWide::kSmemBytes > PairDeep::kSmemBytes ? PairWide::kSmemBytes : PairDeep::kSmemBytes;
-  static std::once_flag attr_once;
-  std::call_once(attr_once, [] {
-    for (auto f : {z4_pair_batch_kernel<kRk4First>, z4_pair_batch_kernel<kRk4Mid>, z4_pair_batch_kernel<kRk4Last>})
-      cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  });
-  const Z4Coef<float> zc = z4_coef<float>(prm);
-  const CUtensorMap* maps = static_cast<const CUtensorMap*>(d_maps);
-  const PairCoef* coefs = static_cast<const PairCoef*>(d_coefs);
-  const dim3 block(32, kPairWarps, 1);
-  switch (rk_form(s)) {
-    case kRk4First:
-      launch_after(z4_pair_batch_kernel<kRk4First>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
-      break;
-    case kRk4Mid:
-      launch_after(z4_pair_batch_kernel<kRk4Mid>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
-      break;
-    case kRk4Last:
-      launch_after(z4_pair_batch_kernel<kRk4Last>, ntiles, block, smem, st, maps, role, d_args, coefs, d_tiles, nwide, s, zc);
-      break;
-    default:
-      return set_error(SF_EINVAL, "batched two-point tiles need the RK4 Kahan forms");
-  }
-  return after_launch("z4_pair_batch_kernel");
 }
 
 }  // namespace sf

@@ -1,10 +1,9 @@
 """Two-point CCZ4 tiles at the edges of their shapes.
 
-Patches of any size on the one-float row offset layout go in tiles of 32 x 8 x 2
-or 16 x 8 x 4 points, whichever covers them with fewer; the padded 96^3-class
-layout in 32 x 16 x 1.  Sizes: one tile, one point less and more along each
+Patches of any size on the one-float row offset layout go in tiles of 32 x 16 x
+1, 32 x 8 x 2 or 16 x 8 x 4 points, whichever covers them in the least time.  Sizes: one tile, one point less and more along each
 axis, odd widths and depths, and sizes that take each shape; through
-sf_substep and through a batch that mixes them.  One RK4 step on NaN-filled
+sf_substep, through a batch that mixes them and through batches of equal patches.  One RK4 step on NaN-filled
 scratch against the FP64 oracle, within the float bound of the 1/dx^2 stencils
 (64 rounding terms of |U| over 12 dx^2, four stages of dt, floor 1e-2); the
 batch gives the same bits as the per-patch launches.
@@ -19,7 +18,7 @@ from paper_1806_04182_gb300.state import PatchState
 
 pytestmark = pytest.mark.gpu
 SIZES = [(3, 3, 3), (16, 8, 4), (15, 7, 3), (17, 9, 5), (32, 8, 2 + 1), (33, 8, 4), (31, 9, 7),
-         (48, 16, 4), (20, 17, 6), (64, 15, 3)]
+         (48, 16, 4), (20, 17, 6), (64, 15, 3), (32, 16, 1 + 2), (36, 41, 5), (33, 17, 3)]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -63,9 +62,10 @@ def test_patch(n):
     assert capi.sf_get_device_status() == capi.SF_OK
 
 
-def test_batch_mixes_shapes():
-    one = [_state(n, q) for q, n in enumerate(SIZES)]
-    many = [_state(n, q) for q, n in enumerate(SIZES)]
+@pytest.mark.parametrize("sizes", [SIZES] + [[n] * 3 for n in ((36, 41, 5), (32, 8, 4), (48, 16, 4))])
+def test_batch(sizes):
+    one = [_state(n, q) for q, n in enumerate(sizes)]
+    many = [_state(n, q) for q, n in enumerate(sizes)]
     b = capi.sf_batch_create(capi.params(), [s.patch(s.B, s.A, s.C) for s, _, _ in many])
     try:
         assert capi.sf_batch_launches_per_step(b) == 4
