@@ -706,7 +706,7 @@ def _amr_rows(hbm_peak: float) -> list[dict]:
     Ub, dxb = inputs.z4_minkowski_noise((96, 96, 96), seed=0, amp=1e-10)
     for lname, lay, kern in (("rows56", dict(x_pitch=56), "one-point TMA tile launch"),
                              ("two_point_layout", dict(x_pitch=56, x_offset=1),
-                              "two-point tile launch (32 x 16 tiles, the second in x half used)")):
+                              "two-point tile launch (16 x 8 x 4 tiles)")):
         level = {}
         for a in range(2):
             for b_ in range(2):

@@ -287,7 +287,7 @@ __device__ __forceinline__ void ssp_write(const PatchArgs<T>& a, const StageArgs
 // below, then the face below the first plane).
 //
 // double is bound by the FP64 pipe (one warp instruction per 16 cycles and
-// SM; 92% of its peak) and reads its stencils from global memory.  float is bound by
+// SM; 86% busy) and reads its stencils from global memory.  float is bound by
 // issue and latency (issue 48%, then fixed-latency waits): its planes are
 // staged in shared memory as field pairs by cp.async, five in a ring, so that
 // a stencil value pair is one 64-bit load with a constant offset.  MR + 1 is
