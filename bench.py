@@ -222,7 +222,7 @@ class NvmlSampler:
 # recorded there (null once the kernel has changed).
 PROFILE = os.path.join(ROOT, "profiles", "z4_pair_fp32dw_96cubed.json")
 KERNEL_SOURCES = ["sf_common.cuh", "sf_dw.cuh", "sf_f2.cuh", "sf_mbar.cuh", "sf_pair.cuh", "sf_z4.cuh",
-                  "sf_z4.cu", "sf_z4_pair.cu"]
+                  "sf_z4.cu", "sf_z4_pair.cuh", "sf_z4_pair.cu"]
 
 
 def kernel_source_hash() -> str:
