@@ -139,13 +139,15 @@ __device__ __forceinline__ double larger(double a, double b) {
 
 // ------------------------------------------------------------ reconstruction
 // Nonlinear weights P_k (without their linear weights) from E_k = eps + beta_k,
-// up to a common factor, and the two reciprocals 1/s_R, 1/s_L.
+// up to a common factor.
 //
 // JS weights are 1/E_k^2; over the common denominator P_0 = (E_1 E_2)^2 and
-// so on.  In float the products E_i E_j are scaled by the power of two of the
-// largest first, so that the largest P_k lies in [1, 4) whatever the units,
-// and E_k is capped at 1.5e19, beyond which its weight is nil (1/E_k^2 is
-// zero in float too).
+// so on, one division fewer.  In float the products E_i E_j are scaled by the
+// power of two of the largest first, so that the largest P_k lies in [1, 4)
+// whatever the units.  Where a product leaves the range of that scale (E_k
+// above 9e18: jumps of 3e9) P_k = (E_min / E_k)^2, in [0, 1], the largest 1; a
+// weight below the range of a float is nil, as 1/E_k^2 is.  (That form for all
+// cells: 1.3% more on the 128^3 step.)
 template <int VAR>
 __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
                                              F2& p1, F2& p2) {
@@ -158,21 +160,27 @@ __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<
     p1 = w(e1);
     p2 = w(e2);
   } else {
-    auto cap = [](F2 e) { return F2(fminf(e.x, 1.5e19f), fminf(e.y, 1.5e19f)); };
-    e0 = cap(e0);
-    e1 = cap(e1);
-    e2 = cap(e2);
     p0 = mul2(e1, e2);
     p1 = mul2(e0, e2);
     p2 = mul2(e0, e1);
-    auto scale = [](float a, float b, float c) {
-      const float m = fmaxf(fmaxf(a, b), c);
-      return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
-    };
-    const F2 sc(scale(p0.x, p1.x, p2.x), scale(p0.y, p1.y, p2.y));
-    p0 = mul2(p0, sc);
-    p1 = mul2(p1, sc);
-    p2 = mul2(p2, sc);
+    auto max3 = [](float a, float b, float c) { return fmaxf(fmaxf(a, b), c); };
+    const float mx = max3(p0.x, p1.x, p2.x), my = max3(p0.y, p1.y, p2.y);
+    if (fmaxf(mx, my) < 0x1p126f) {
+      auto scale = [](float m) { return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000)); };
+      const F2 sc(scale(mx), scale(my));
+      p0 = mul2(p0, sc);
+      p1 = mul2(p1, sc);
+      p2 = mul2(p2, sc);
+    } else {
+      const float lx = fminf(fminf(e0.x, e1.x), e2.x), ly = fminf(fminf(e0.y, e1.y), e2.y);
+      auto w = [&](F2 e) {
+        const F2 z = nrecip2(e);  // (E_k infinite: NaN, which the saturation takes to 0)
+        return F2(__saturatef(-lx * z.x), __saturatef(-ly * z.y));
+      };
+      p0 = w(e0);
+      p1 = w(e1);
+      p2 = w(e2);
+    }
     p0 = mul2(p0, p0);
     p1 = mul2(p1, p1);
     p2 = mul2(p2, p2);

@@ -69,3 +69,12 @@ def _check(U, dx, precision, **kw):
 def test_jump(n, axis, variant, J, precision):
     U = _states(n, axis, J, seed=axis)
     _check(U, tuple(1.0 / v for v in n), precision, weno_variant=variant)
+
+
+# the smoothness indicators are squares of up to 1e12, their products of squares
+# beyond a float
+@pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
+@pytest.mark.parametrize("n,axis", [((40, 9, 5), 0), ((34, 18, 4), 1), ((9, 8, 16), 2)])
+@pytest.mark.parametrize("J", [4e9, 1e12])
+def test_js_range(n, axis, J, precision):
+    _check(_states(n, axis, J, seed=axis), tuple(1.0 / v for v in n), precision, weno_variant=0)
