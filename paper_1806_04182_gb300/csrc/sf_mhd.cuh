@@ -148,6 +148,10 @@ __device__ __forceinline__ double larger(double a, double b) {
 // above 9e18: jumps of 3e9) P_k = (E_min / E_k)^2, in [0, 1], the largest 1; a
 // weight below the range of a float is nil, as 1/E_k^2 is.  (That form for all
 // cells: 1.3% more on the 128^3 step.)
+// 2^-floor(log2 m) of a normal m < 2^127
+__device__ __forceinline__ float inv_pow2(float m) {
+  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+}
 template <int VAR>
 __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
                                              F2& p1, F2& p2) {
@@ -166,8 +170,7 @@ __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<
     auto max3 = [](float a, float b, float c) { return fmaxf(fmaxf(a, b), c); };
     const float mx = max3(p0.x, p1.x, p2.x), my = max3(p0.y, p1.y, p2.y);
     if (fmaxf(mx, my) < 0x1p126f) {
-      auto scale = [](float m) { return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000)); };
-      const F2 sc(scale(mx), scale(my));
+      const F2 sc(inv_pow2(mx), inv_pow2(my));
       p0 = mul2(p0, sc);
       p1 = mul2(p1, sc);
       p2 = mul2(p2, sc);
@@ -243,9 +246,15 @@ __device__ __forceinline__ void weno_edges(const P* w, T eps, const MhdCoef<T>& 
   if constexpr (VAR == 2) {
     const P ep(eps);
     P e0 = fma2(d2, d2, ep), e1 = fma2(d1, d1, ep);
-    if constexpr (sizeof(T) == 4) {  // as weno_weights: beyond the cap the weight is nil
-      e0 = P(fminf(e0.x, 1.5e19f), fminf(e0.y, 1.5e19f));
-      e1 = P(fminf(e1.x, 1.5e19f), fminf(e1.y, 1.5e19f));
+    if constexpr (sizeof(T) == 4) {
+      // scaled so that the larger one lies in [1, 2): the squares and their
+      // products with the differences stay in range (capped: 1.5e38 < 2^127)
+      auto cap = [](P e) { return P(fminf(e.x, 1.5e38f), fminf(e.y, 1.5e38f)); };
+      e0 = cap(e0);
+      e1 = cap(e1);
+      const P sc(inv_pow2(fmaxf(e0.x, e1.x)), inv_pow2(fmaxf(e0.y, e1.y)));
+      e0 = mul2(e0, sc);
+      e1 = mul2(e1, sc);
     }
     const P p0 = mul2(e1, e1), p1 = mul2(e0, e0);
     // er = w_2 + (2 p0 d2 + p1 d1) / (2 (2 p0 + p1)), el its mirror image

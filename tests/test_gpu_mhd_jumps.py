@@ -78,3 +78,11 @@ def test_jump(n, axis, variant, J, precision):
 @pytest.mark.parametrize("J", [4e9, 1e12])
 def test_js_range(n, axis, J, precision):
     _check(_states(n, axis, J, seed=axis), tuple(1.0 / v for v in n), precision, weno_variant=0)
+
+
+# the weights' products with the differences go with the fifth power of a jump
+@pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
+@pytest.mark.parametrize("n,axis", [((40, 9, 5), 0), ((34, 18, 4), 1), ((9, 8, 16), 2)])
+@pytest.mark.parametrize("J", [1e8, 4e9, 1e12])
+def test_weno3_range(n, axis, J, precision):
+    _check(_states(n, axis, J, seed=axis), tuple(1.0 / v for v in n), precision, weno_variant=2)
