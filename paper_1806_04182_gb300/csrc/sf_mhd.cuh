@@ -156,13 +156,20 @@ template <int VAR>
 __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
                                              F2& p1, F2& p2) {
   if constexpr (VAR == 1) {
+    // 1 + (tau / E_k)^q, times the q-th power of a scale: beyond ratios of 2^30
+    // (a jump of 2 beside a uniform state on 128 cells) the inverse power of
+    // two of the largest, so that the weights and their sums stay in range
     const F2 tau = abs2(sub2(e0, e2));
-    auto w = [&](F2 e) {
-      return F2(1.0f + wz_pow(tau.x / e.x, mc.q), 1.0f + wz_pow(tau.y / e.y, mc.q));
+    auto lane = [&](float t, float a, float b, float c, float& pa, float& pb, float& pc) {
+      auto ratio = [&](float e) { return fminf(t / e, 1.5e38f); };
+      const float ra = ratio(a), rb = ratio(b), rc = ratio(c), m = fmaxf(fmaxf(ra, rb), rc);
+      const float u = m < 0x1p30f ? 1.0f : inv_pow2(m), one = wz_pow(u, mc.q);
+      pa = one + wz_pow(ra * u, mc.q);
+      pb = one + wz_pow(rb * u, mc.q);
+      pc = one + wz_pow(rc * u, mc.q);
     };
-    p0 = w(e0);
-    p1 = w(e1);
-    p2 = w(e2);
+    lane(tau.x, e0.x, e1.x, e2.x, p0.x, p1.x, p2.x);
+    lane(tau.y, e0.y, e1.y, e2.y, p0.y, p1.y, p2.y);
   } else {
     p0 = mul2(e1, e2);
     p1 = mul2(e0, e2);

@@ -86,3 +86,13 @@ def test_js_range(n, axis, J, precision):
 @pytest.mark.parametrize("J", [1e8, 4e9, 1e12])
 def test_weno3_range(n, axis, J, precision):
     _check(_states(n, axis, J, seed=axis), tuple(1.0 / v for v in n), precision, weno_variant=2)
+
+
+# WENO-Z: the ratio of the indicators beside a jump is its square over epsilon
+# where the state is uniform; its q-th power leaves a float from jumps of 1e5 on
+@pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
+@pytest.mark.parametrize("n,axis", [((40, 9, 5), 0), ((34, 18, 4), 1), ((9, 8, 16), 2)])
+@pytest.mark.parametrize("J,noise,q", [(1e6, 0.0, 2.0), (1e6, 0.0, 1.5), (1e8, 0.1, 2.0), (1e12, 0.1, 2.0)])
+def test_z_range(n, axis, J, noise, q, precision):
+    U = _states(n, axis, J, seed=axis, noise=noise)
+    _check(U, tuple(1.0 / v for v in n), precision, weno_variant=1, weno_q=q)
