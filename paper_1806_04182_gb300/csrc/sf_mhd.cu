@@ -231,8 +231,7 @@ __device__ __forceinline__ double cell_rate(const double* q, const MhdCoef<doubl
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
     const double disc = __fma_rn(n2, bb[d], hh);
-    const bool below = (unsigned)__double2hiint(disc) - 0x80000000u < 0x7ff00000u;  // finite, < 0
-    const double cf = sqrt1(__dadd_rn(sqrt1(below ? 0.0 : disc), h));
+    const double cf = sqrt1(nonneg(__dadd_rn(sqrt1(nonneg(disc)), h)));
     rate = fmax(rate, __dmul_rn(__dadd_rn(fabs(nv[d]), cf), mc.idx[d]));  // NaN kept out
   }
   return rate;

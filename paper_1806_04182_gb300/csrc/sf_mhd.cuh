@@ -128,6 +128,18 @@ __device__ __forceinline__ F2 pos2(F2 x) { return F2(fmaxf(x.x, 0.0f), fmaxf(x.y
 __device__ __forceinline__ R2 pos2(R2 x) {
   return R2(__double2hiint(x.x) < 0 ? 0.0 : x.x, __double2hiint(x.y) < 0 ? 0.0 : x.y);
 }
+// the same, but NaN stays (the sum under the root of the signal speed: of a
+// state with negative pressure it is a rounding error of either sign)
+__device__ __forceinline__ float nonneg(float x) {
+  float r;
+  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ double nonneg(double x) {
+  return (unsigned)__double2hiint(x) - 0x80000000u < 0x7ff00000u ? 0.0 : x;  // finite, < 0
+}
+__device__ __forceinline__ F2 nonneg2(F2 x) { return F2(nonneg(x.x), nonneg(x.y)); }
+__device__ __forceinline__ R2 nonneg2(R2 x) { return R2(nonneg(x.x), nonneg(x.y)); }
 __device__ __forceinline__ F2 abs2(F2 x) { return F2(fabsf(x.x), fabsf(x.y)); }
 __device__ __forceinline__ R2 abs2(R2 x) { return R2(fabs(x.x), fabs(x.y)); }
 // the larger of two non-negative values; double: as integers (their bits are
@@ -321,7 +333,7 @@ __device__ __forceinline__ void llf_flux2(const P* q, T gamma, T* F) {
   const P na2 = mul2(mul2(P(gamma), pr), nir);
   const P h = mul2(P(T(-0.5)), fma2(B2, nir, na2));
   const P disc = fma2(neg2(na2), mul2(bd2, nir), mul2(h, h));
-  const P cf = sqrt2(add2(sqrt2(pos2(disc)), h));
+  const P cf = sqrt2(nonneg2(add2(sqrt2(pos2(disc)), h)));
   const T S = larger(fabs(nv[D].x) + cf.x, fabs(nv[D].y) + cf.y);
   auto out = [&](int f, P nf) { F[f] = fma(-S, q[f].y - q[f].x, -nf.x - nf.y); };
   F[0] = fma(-S, q[0].y - q[0].x, Sd.x + Sd.y);

@@ -46,7 +46,7 @@ def _local(a):
     return m
 
 
-def _check(U, dx, precision, **kw):
+def _check(U, dx, precision, speed_err=0.0, **kw):
     n = U.shape[:0:-1]
     eps = float(np.finfo(np.float64 if precision == capi.SF_FP64 else np.float32).eps)
     if precision != capi.SF_FP64:
@@ -56,7 +56,7 @@ def _check(U, dx, precision, **kw):
     got = st.rhs().double().cpu().numpy()
     want = oracle.rhs(oracle.MHD, oracle.ghosted(U.copy()), dx, oracle.params(**kw))
     hydro, mag = (_local(np.abs(U[a]).max(0)) for a in (slice(0, 5), slice(5, 8)))
-    tol = (40 if precision == capi.SF_FP64 else 20) * eps * 3 * sum(2 / h for h in dx)
+    tol = ((40 if precision == capi.SF_FP64 else 20) * eps * 3 + 0.5 * speed_err) * sum(2 / h for h in dx)
     for f in range(8):
         e = np.abs(got[f] - want[f]) / (tol * (hydro if f < 5 else mag))
         assert np.isfinite(e).all() and e.max() < 1, (f, np.nanmax(e), np.isnan(e).sum())
@@ -96,3 +96,42 @@ def test_weno3_range(n, axis, J, precision):
 def test_z_range(n, axis, J, noise, q, precision):
     U = _states(n, axis, J, seed=axis, noise=noise)
     _check(U, tuple(1.0 / v for v in n), precision, weno_variant=1, weno_q=q)
+
+
+# Negative gas pressure p and no field along x and y: s = (gamma p + B^2) / rho
+# is negative, s + sqrt(s^2) zero, and the signal speed |v_d|; rounding leaves
+# up to 2 eps |s| of the sum, a speed of its root.
+def _negative_pressure(n, seed, noise, vx=0.0):
+    r = np.random.default_rng(seed).uniform(-noise, noise, (5, n[2], n[1], n[0]))
+    zero = np.zeros(r.shape[1:])
+    rho, p = 1 + r[0], -0.5 + 0.5 * r[4]
+    U = inputs.mhd_primitive_to_conserved(rho, [vx + r[1], r[2], r[3]], p, [zero, zero, zero + 0.2], 5 / 3)
+    return U, float(np.abs((5 / 3 * p + 0.04) / rho).max())
+
+
+@pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
+@pytest.mark.parametrize("n", [(40, 9, 5), (9, 8, 16)])
+def test_negative_pressure(n, precision):
+    U, s = _negative_pressure(n, 3, 0.1)
+    eps = float(np.finfo(np.float64 if precision == capi.SF_FP64 else np.float32).eps)
+    _check(U, tuple(1.0 / v for v in n), precision, speed_err=np.sqrt(2 * eps * 1.5 * s))
+
+
+@pytest.mark.parametrize("precision", [capi.SF_FP64, capi.SF_FP32_BULK])
+@pytest.mark.parametrize("fused", [False, True])
+def test_negative_pressure_rate(fused, precision):
+    """Uniform states, one after the other, moving along x: the rate is |v_x| / dx."""
+    n, dx = (3, 3, 3), (0.25, 0.25, 0.25)
+    eps = float(np.finfo(np.float64 if precision == capi.SF_FP64 else np.float32).eps)
+    for seed in range(24):
+        vx = 1.5 + 0.01 * seed
+        U, s = _negative_pressure((1, 1, 1), seed, 0.3, vx)
+        vx = (U[1] / U[0]).item()
+        st = PatchState(capi.SF_MHD, n, dx, 1e-3, precision=precision, prm=capi.params(rk=capi.SF_SSPRK3))
+        st.upload(np.broadcast_to(U, (8,) + n[::-1]).copy())
+        if fused:  # the rate of the state after a step, which is the same state
+            rate = torch.zeros(1, dtype=torch.float64, device="cuda")
+            st._steps(1, torch.cuda.current_stream().cuda_stream, rate=rate.data_ptr())
+        else:
+            rate = st.mhd_max_rate()
+        assert abs(rate.item() * dx[0] - vx) < 16 * eps * vx + np.sqrt(2 * eps * s), (seed, rate.item())
