@@ -640,10 +640,13 @@ __global__ void __launch_bounds__(MX * (MR + 1), 16 / (MR + 1))
 // row ty + 1 (shared memory), and carries the z-face below the current plane
 // in registers while it marches mz planes (a first pass evaluates only the
 // z-face below the first plane).  The three directions run in one rolled
-// loop, so the kernel holds one copy of the face code.
+// loop, so the kernel holds one copy of the face code.  One block per SM is
+// asked for (without that the compiler halves the reads in flight of float
+// WENO5: 20^3 WENO-Z step 413 against 430 us), two for float WENO3, which fits
+// in 128 registers (110 x 30 x 70 step 467 -> 319 us).
 constexpr int SY = 8;
 template <typename T, int VAR>
-__global__ void __launch_bounds__(MX * SY)
+__global__ void __launch_bounds__(MX * SY, sizeof(T) == 4 && VAR == 2 ? 2 : 1)
     mhd_split_kernel(PatchArgs<T> a, StageArgs s, MhdCoef<T> mc, int mz) {
   __shared__ T fy[SY][MX][8];
   wait_predecessor();
