@@ -44,6 +44,15 @@ unsigned int* status_ptr() {
   return cache[dev];
 }
 
+int sm_count() {
+  static int cache[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+  if (!cache[dev] && cudaDeviceGetAttribute(&cache[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    cache[dev] = 0;
+  return cache[dev];
+}
+
 void normalise_strides(sf_patch& p, int nf) {
   (void)nf;
   const long long g2 = 2LL * p.ghost;

@@ -227,17 +227,18 @@ sf_status build_pair(sf_batch* b) {
   const size_t cb = z4_pair_coef_bytes();
   std::vector<unsigned char> maps((size_t)6 * b->npatch * kTmaMapBytes, 0), coefs(cb * b->npatch, 0);
   std::vector<TmaTile> lists[3];
-  int only = -1;  // the one shape that all patches take, 3 if they differ
-  for (const sf_patch& p : b->patches) {
-    if (!z4_pair_batch_eligible(b->prm, p)) continue;
-    const int w = z4_pair_shape(p, 0);
-    only = only < 0 || only == w ? w : 3;
-  }
-  for (int q = 0; q < b->npatch; ++q) {
-    const sf_patch& p = b->patches[q];
-    if (!z4_pair_batch_eligible(b->prm, p)) continue;
+  std::vector<const sf_patch*> elig;
+  std::vector<int> index, shapes;
+  for (int q = 0; q < b->npatch; ++q)
+    if (z4_pair_batch_eligible(b->prm, b->patches[q])) {
+      elig.push_back(&b->patches[q]);
+      index.push_back(q);
+    }
+  z4_pair_batch_shapes(elig, shapes);
+  for (size_t m = 0; m < elig.size(); ++m) {
+    const sf_patch& p = *elig[m];
+    const int q = index[m], w = shapes[m];
     b->pair[q] = 1;
-    const int w = only < 3 ? only : z4_pair_shape(p, 1);
     sf_status e = encode_z4_pair_batch(maps.data() + (size_t)6 * q * kTmaMapBytes, coefs.data() + cb * q,
                                        b->prm, p, w);
     if (e) return e;

@@ -1,6 +1,8 @@
 // Internal declarations shared by the translation units of libsf.so.
 #pragma once
 
+#include <vector>
+
 #include "sf_common.cuh"
 
 namespace sf {
@@ -10,6 +12,8 @@ sf_status set_error(sf_status code, const char* fmt, ...);
 sf_status after_launch(const char* what);
 // device address of the status word on the current device (nullptr if none)
 unsigned int* status_ptr();
+// SMs of the current device (0 if none)
+int sm_count();
 
 // per-system stage launchers; rhs_out != nullptr selects "RHS only" output
 sf_status launch_wave(const sf_params& prm, const sf_patch& p, const StageArgs& s, int stage,
@@ -49,7 +53,8 @@ bool z4_tma_batch_eligible(const sf_params& prm, const sf_patch& p);
 // boxes of the u_n, u_stage, u_next roles, for the patch's shape) and the
 // patch's stencil weights (z4_pair_coef_bytes each) in device memory.
 constexpr int kPairShapes[3][3] = {{32, 16, 1}, {32, 8, 2}, {16, 8, 4}};
-int z4_pair_shape(const sf_patch& p, int first);  // the shape from `first` on that covers p in the least time
+int z4_pair_shape(const sf_patch& p);  // of a launch over p alone
+void z4_pair_batch_shapes(const std::vector<const sf_patch*>& ps, std::vector<int>& shapes);
 bool z4_pair_batch_eligible(const sf_params& prm, const sf_patch& p);
 size_t z4_pair_coef_bytes();
 sf_status encode_z4_pair_batch(void* maps6, void* coef, const sf_params& prm, const sf_patch& p, int w);

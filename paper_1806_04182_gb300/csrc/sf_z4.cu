@@ -49,15 +49,6 @@ __global__ void __launch_bounds__(128, MINB)
   write_fields<T, 25>(a, s, im, c, i, j, k, rbuf + tid, 128);
 }
 
-static int sm_count() {
-  static int cache[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
-  if (!cache[dev] && cudaDeviceGetAttribute(&cache[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-    cache[dev] = 0;
-  return cache[dev];
-}
-
 template <typename T, typename H, int MINB>
 static void launch_kernel(const PatchArgs<T>& a, const StageArgs& s, const sf_params& prm, const sf_patch& p,
                           dim3 grid, cudaStream_t st) {

@@ -7,25 +7,70 @@
 // (kPairShapes).  Lanes outside the patch idle: with 32 x 16 x 1 tiles alone,
 // 36% of them on patches of 16 to 64 points a side and 25% on 48^3 (96 mixed
 // patches 11.6 ms per RK4 step, eight 48^3 patches with halo exchange 1.59; with
-// the other two alone 10.0 and 1.36).  A tile of two or four planes takes some
-// 15% or 20% longer than a flat one (96^3, which all three cover exactly), so a
-// patch takes the shape with the least tiles x time (four 36 x 41 x 17 patches:
-// 400 us a step with the other two, 336 with all three).
+// the other two alone 10.0 and 1.36).  A launch takes rounds of one tile per
+// SM, and a round of the three shapes 23.9, 24.4 and 25.5 us a stage, so a patch
+// takes the shape of the least rounds x time.  Stage of 80 x 24 x 23 (138, 108
+// or 90 tiles: one round) 23.9, 24.0, 25.1 us; 48^3 (two rounds) 47.5, 48.4,
+// 51.7; 60 x 20 x 88 (3, 2, 2) 69, 50, 55; 70 x 50 x 61 (5, 5, 4) 113, 107, 96.
+// (By tiles x time instead the first two took the deep tiles.)
+#include <algorithm>
+
 #include "sf_z4_pair.cuh"
 
 namespace sf {
 
-int z4_pair_shape(const sf_patch& p, int first) {
-  auto tiles = [&](const int* t) {
-    long long n = 1;
-    for (int d = 0; d < 3; ++d) n *= (p.n[d] + t[d] - 1) / t[d];
-    return n;
-  };
-  constexpr int time[3] = {20, 23, 24};
-  int best = first;
-  for (int w = first + 1; w < 3; ++w)
-    if (tiles(kPairShapes[w]) * time[w] < tiles(kPairShapes[best]) * time[best]) best = w;
+constexpr int kPairTime[3] = {40, 41, 43};  // of a round, relative
+static long long pair_tiles(const sf_patch& p, int w) {
+  long long n = 1;
+  for (int d = 0; d < 3; ++d) n *= (p.n[d] + kPairShapes[w][d] - 1) / kPairShapes[w][d];
+  return n;
+}
+static long long pair_rounds(long long tiles) {
+  const long long sms = std::max(1, sm_count());
+  return (tiles + sms - 1) / sms;
+}
+
+int z4_pair_shape(const sf_patch& p) {
+  int best = 0;
+  long long cost = -1;
+  for (int w = 0; w < 3; ++w) {
+    const long long c = pair_rounds(pair_tiles(p, w)) * kPairTime[w];
+    if (cost < 0 || c < cost) {
+      cost = c;
+      best = w;
+    }
+  }
   return best;
+}
+
+// The tiles of all patches of a launch share its rounds: one shape for all, or
+// the wide or the deep one for each patch by its tiles x time.
+void z4_pair_batch_shapes(const std::vector<const sf_patch*>& ps, std::vector<int>& shapes) {
+  shapes.assign(ps.size(), 0);
+  if (ps.empty()) return;
+  double cost = 0.0;
+  int best = 0;
+  for (int w = 0; w < 3; ++w) {
+    long long n = 0;
+    for (const sf_patch* p : ps) n += pair_tiles(*p, w);
+    const double c = (double)(pair_rounds(n) * kPairTime[w]);
+    if (w == 0 || c < cost) {
+      cost = c;
+      best = w;
+    }
+  }
+  std::vector<int> mixed(ps.size());
+  long long n = 0, work = 0;
+  for (size_t q = 0; q < ps.size(); ++q) {
+    const long long t1 = pair_tiles(*ps[q], 1), t2 = pair_tiles(*ps[q], 2);
+    mixed[q] = t2 * kPairTime[2] < t1 * kPairTime[1] ? 2 : 1;
+    n += mixed[q] == 2 ? t2 : t1;
+    work += std::min(t2 * kPairTime[2], t1 * kPairTime[1]);
+  }
+  if ((double)pair_rounds(n) * (double)work / (double)n < cost)
+    shapes = mixed;
+  else
+    shapes.assign(ps.size(), best);
 }
 
 // One CTA per tile of one patch (the RK4 Kahan forms).
@@ -87,7 +132,7 @@ bool z4_pair_any_eligible(const sf_params& prm, const sf_patch& p, const StageAr
 
 sf_status launch_z4_pair_any(const sf_params& prm, const sf_patch& p, const StageArgs& s, int stage,
                              cudaStream_t st) {
-  switch (z4_pair_shape(p, 0)) {
+  switch (z4_pair_shape(p)) {
     case 0: return launch_any<PairFlat>(prm, p, s, stage, st);
     case 1: return launch_any<PairWide>(prm, p, s, stage, st);
     default: return launch_any<PairDeep>(prm, p, s, stage, st);
