@@ -11,6 +11,7 @@ SSP-RK3: stage 0: A -> B, 1: B -> C, 2: C -> A.
 """
 from __future__ import annotations
 
+import ctypes
 import json
 import struct
 
@@ -26,6 +27,20 @@ def _stream_handle(stream) -> int:
     if isinstance(stream, torch.cuda.Stream):
         return stream.cuda_stream
     return int(stream)
+
+
+def _packer(cls) -> struct.Struct:
+    """A ctypes structure's layout as a Struct, one value per element of its
+    fields in their order."""
+    codes = {ctypes.c_int32: "i", ctypes.c_double: "d", ctypes.c_int64: "q", ctypes.c_void_p: "Q"}
+    fmt = ""
+    for _, t in cls._fields_:
+        base, count = getattr(t, "_type_", t), getattr(t, "_length_", 1)
+        fmt += codes[base if count > 1 else t] * count
+    packer = struct.Struct("=" + fmt)
+    if packer.size != ctypes.sizeof(cls):
+        raise TypeError(f"{cls.__name__} has padding")
+    return packer
 
 
 class PatchState:
@@ -193,9 +208,11 @@ class PatchState:
 
     # sf_patch and sf_state as bytes, in the order of their fields (one pack call
     # instead of an attribute assignment per field: a step of a small patch
-    # takes less time on the GPU than its descriptors took to fill)
-    _GEOM = struct.Struct("=4i4d2i3q6Q")
-    _STATE = struct.Struct("=5Q")
+    # takes less time on the GPU than its descriptors took to fill).  The
+    # formats are read off the structures: a field added to one of them is a
+    # value missing from its pack call.
+    _GEOM = _packer(capi.sf_patch)
+    _STATE = _packer(capi.sf_state)
 
     def _steps(self, nsteps: int, h: int, adjoint: bool = False, rate: int = 0) -> None:
         g = capi.sf_patch.from_buffer_copy(self._GEOM.pack(
