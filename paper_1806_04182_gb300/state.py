@@ -215,6 +215,8 @@ class PatchState:
     _STATE = _packer(capi.sf_state)
 
     def _steps(self, nsteps: int, h: int, adjoint: bool = False, rate: int = 0) -> None:
+        if nsteps <= 0:
+            return
         g = capi.sf_patch.from_buffer_copy(self._GEOM.pack(
             *self.n, self.g, *self.dx, self.dt, self.system, self.precision, *self.strides,
             0, 0, 0, 0, 0, rate))

@@ -49,3 +49,11 @@ def test_padding():
     pad = type("pad", (ctypes.Structure,), {"_fields_": [("a", ctypes.c_int32), ("b", ctypes.c_double)]})
     with pytest.raises(TypeError):
         state._packer(pad)
+
+
+@pytest.mark.parametrize("n", [0, -1])
+def test_no_steps(n):
+    """No step, no call: a patch that sf_steps would refuse included."""
+    st = PatchState(capi.SF_WAVE, (2, 2, 2), (0.1, 0.1, 0.1), 0.01, device="cpu")
+    st.step(n, stream=0)
+    st.adjoint_step(n, stream=0)
