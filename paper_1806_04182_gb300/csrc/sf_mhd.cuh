@@ -12,9 +12,9 @@
 // plus the weighted corrections, so a uniform state is reproduced exactly.
 // Each correction holds only differences of its own stencil: a jump enters
 // through the stencils that its weights switch off and nowhere else.  (With
-// d_2/2 taken out of the three, five operations fewer, a jump J beside the cell
+// d_2/2 taken out of the three, two operations fewer, a jump J beside the cell
 // had to cancel against it and left an error of eps J: float edge values wrong
-// by 14% beside a jump by 10^6, now by 1e-7.)  46 operations give both edges
+// by 14% beside a jump by 10^6, now by 1e-7.)  43 operations give both edges
 // (double) (App. B evaluated per face and per side takes about 124 for the
 // same two values).
 #pragma once
@@ -295,16 +295,16 @@ __device__ __forceinline__ void weno_edges(const P* w, T eps, const MhdCoef<T>& 
   const P e2 = fma2(a2, fma2(c43, a2, d1), g1);
   P p0, p1, p2;
   weno_weights<VAR>(e0, e1, e2, mc, p0, p1, p2);
-  // right edge: weights 3 p0, 6 p1, p2; left edge: p0, 6 p1, 3 p2
+  // right edge: weights 3 p0, 6 p1, p2; left edge: p0, 6 p1, 3 p2.  The weighted
+  // corrections x 6 (left edge with opposite sign), 4 d_2 - d_3 = 3 d_2 - a_0 and
+  // so on, grouped by difference: a factor of d_k or a_k holds the weights of
+  // the stencils that contain it and no others
   const P two(T(2)), three(T(3)), ct(T(2.0 / 3.0));
-  const P h1 = add2(p1, p1);
-  const P sr = fma2(three, add2(p0, h1), p2), sl = fma2(three, add2(p2, h1), p0);
-  // the candidates' corrections x 6 (left edge with opposite sign), 4 d_2 - d_3
-  // = 3 d_2 - a_0 and so on; those of weight 1 a third of it
-  const P r0 = fma2(three, d2, neg2(a0)), r1 = fma2(two, d2, d1), r2 = fma2(ct, a2, d1);
-  const P l2 = fma2(three, d1, a2), l1 = fma2(two, d1, d2), l0 = fma2(ct, neg2(a0), d2);
-  const P nr = fma2(p0, r0, fma2(h1, r1, mul2(p2, r2)));
-  const P nl = fma2(p2, l2, fma2(h1, l1, mul2(p0, l0)));
+  const P p01 = fma2(two, p1, p0), p12 = fma2(two, p1, p2);
+  const P sr = fma2(three, p01, p2), sl = fma2(three, p12, p0);
+  const P qa = mul2(p0, a0), qc = mul2(p2, a2);
+  const P nr = fma2(d2, fma2(two, p01, p0), fma2(d1, p12, fma2(ct, qc, neg2(qa))));
+  const P nl = fma2(d1, fma2(two, p12, p2), fma2(d2, p01, fma2(neg2(ct), qa, qc)));
   P ir, il;
   half_recips<VAR>(sr, sl, ir, il);
   er = fma2(neg2(nr), ir, w[2]);
