@@ -41,28 +41,6 @@
 namespace sf {
 namespace {
 
-// mbar_wait of sf_mbar.cuh with its loop in C++: larger code, but these kernels
-// have room (121 KB of 128) and the hand-written loop, which keeps every lane's
-// result, costs them 1 to 3% (59 x 46 x 53 step 251 against 258 us).
-__device__ __forceinline__ bool ring_wait(uint64_t* b, unsigned parity, long long limit) {
-  auto done = [&] {
-    unsigned ok;
-    asm volatile(
-        "{\n .reg .pred p;\n"
-        " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(saddr(b)), "r"(parity)
-        : "memory");
-    return ok != 0;
-  };
-  if (done()) return true;
-  const long long t0 = clock64();
-  while (!done())
-    if (clock64() - t0 > limit) return false;
-  return true;
-}
-
 // A CTA computes an XP x BY x 1 tile of points (32 / XP rows per warp: one
 // row of 32 points, or two rows of 16); the staged box of a field is
 // XB x (BY + 6) x TZ floats with XB = XP + 6 rounded up to 16 bytes, each slot
@@ -151,7 +129,7 @@ struct TmaSrc {
   // (use j - kSlots) has been released by every warp
   __device__ __forceinline__ void issue(int j) {
     const int sl = j % kSlots;
-    if (j >= kSlots && !dead) dead = !ring_wait(&empty[sl], ((j / kSlots) - 1) & 1, kWaitCycles);
+    if (j >= kSlots && !dead) dead = !mbar_wait(&empty[sl], ((j / kSlots) - 1) & 1, kWaitCycles);
     if (dead) return;
     mbar_expect(&full[sl], kBoxBytes);
     tma_load_4d(tiles + sl * kSlotFloats, map, gx, gy, gz, tma_field(j), &full[sl]);
@@ -171,7 +149,7 @@ struct TmaSrc {
       if (lane0) mbar_arrive(&empty[(i - 1) % kSlots]);
     }
     cur = i % kSlots;
-    if (!dead) dead = !ring_wait(&full[cur], (i / kSlots) & 1, kWaitCycles);
+    if (!dead) dead = !mbar_wait(&full[cur], (i / kSlots) & 1, kWaitCycles);
   }
 
   // the leader's warp consumed every load it issued unless a wait gave up;
@@ -179,7 +157,7 @@ struct TmaSrc {
   __device__ __forceinline__ void finish() {
     if (dead) atomicOr(status, ST_TIMEOUT);
     if (leader && dead)
-      for (int j = use; j < issued; ++j) ring_wait(&full[j % kSlots], (j / kSlots) & 1, kWaitCycles);
+      for (int j = use; j < issued; ++j) mbar_wait(&full[j % kSlots], (j / kSlots) & 1, kWaitCycles);
   }
 };
 
