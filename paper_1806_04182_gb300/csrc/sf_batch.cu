@@ -124,7 +124,7 @@ struct sf_batch {
   int2* d_shape = nullptr;
   Item* d_items = nullptr;
   int nitems = 0;
-  bool wave_items = false;  // all of them wave items
+  bool wave_items = false;  // all of the batch's are wave items
   unsigned int* d_counter = nullptr;
   std::vector<char> tma;  // patch q goes to the TMA-staged CCZ4 kernel
   std::vector<char> pair;  // patch q goes to the two-point CCZ4 kernel (takes precedence)
@@ -184,6 +184,7 @@ sf_status upload_args(sf_batch* b) {
 sf_status build_items(sf_batch* b, int only_class) {
   std::vector<Item> items;
   std::vector<int2> shapes(b->npatch);
+  bool z4_items = false;  // of any class: which kernel the batch runs is fixed while a class is tuned
   for (int pass = 0; pass < 2; ++pass)
     for (int q = 0; q < b->npatch; ++q) {
       const sf_patch& p = b->patches[q];
@@ -191,6 +192,7 @@ sf_status build_items(sf_batch* b, int only_class) {
       if ((pass == 0) != z4) continue;
       if (!b->tma.empty() && b->tma[q]) continue;
       if (!b->pair.empty() && b->pair[q]) continue;
+      z4_items = z4_items || z4;
       const int cls = class_of(p);
       const Shape sh = kShapes[b->shape_of_class[cls]];
       shapes[q] = make_int2(sh.tx, sh.tz);
@@ -202,7 +204,7 @@ sf_status build_items(sf_batch* b, int only_class) {
   if (b->d_items) cudaFree(b->d_items);
   b->d_items = nullptr;
   b->nitems = (int)items.size();
-  b->wave_items = !items.empty() && b->patches[items[0].patch].system != SF_Z4;  // CCZ4 items come first
+  b->wave_items = !items.empty() && !z4_items;
   if (!items.empty()) {
     if (cudaMalloc(&b->d_items, items.size() * sizeof(Item)) != cudaSuccess)
       return set_error(SF_ECUDA, "batch: cudaMalloc of work list failed");
