@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(256) copy_boxes_kernel(BoxBatch bb) {
       const long long si = b.src_off + f * b.src_sf + (long long)z * b.src_step * b.src_sz +
                            (long long)y * b.src_step * b.src_sy + (long long)x * b.src_step;
       d[u] = b.dst_off + f * b.dst_sf + (long long)z * b.dst_sz + (long long)y * b.dst_sy + x;
-      v[u] = __ldg(src + si);
+      v[u] = src[si];
     }
 #pragma unroll
     for (int u = 0; u < kCopyIlp; ++u)
@@ -123,11 +123,11 @@ struct Combo {
 // accuracy, and the combination and interpolation weights sum to one.
 template <typename T, int NS>
 __device__ __forceinline__ T node_value(const Combo<T>& cb, long long o) {
-  T v = __ldg(cb.s[0] + o);
+  T v = cb.s[0][o];
   if (NS > 0) {
     const T u = v;
 #pragma unroll
-    for (int m = 1; m <= NS; ++m) v += cb.c[m - 1] * (__ldg(cb.s[m] + o) - u);
+    for (int m = 1; m <= NS; ++m) v += cb.c[m - 1] * (cb.s[m][o] - u);
   }
   return v;
 }

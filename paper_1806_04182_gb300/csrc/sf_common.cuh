@@ -27,8 +27,8 @@ struct PatchArgs {
   int g;
   long long sy, sz, sf;
   long long ninterior;
-  const T* __restrict__ us;  // stage input (ghosted)
-  const T* __restrict__ un;  // U^n (ghosted)
+  const T* us;  // stage input (ghosted)
+  const T* un;  // U^n (ghosted)
   T* acc;
   T* nx;                     // next stage / U^{n+1}, or the RHS output (unghosted)
   T* kh;
@@ -66,43 +66,6 @@ struct StageArgs {
   int check_finite;
   unsigned int* status;  // device status word
 };
-
-// ------------------------------------------------------------ stencils
-// Sec. II.B.1.  `p` points at the centre value, `s` is the element stride
-// of the direction.
-template <typename T>
-__device__ __forceinline__ T d1(const T* __restrict__ p, long long s, T i12h) {
-  return ((__ldg(p - 2 * s) - __ldg(p + 2 * s)) + T(8) * (__ldg(p + s) - __ldg(p - s))) * i12h;
-}
-
-template <typename T>
-__device__ __forceinline__ T d2(const T* __restrict__ p, long long s, T c0, T i12h2) {
-  return (T(16) * (__ldg(p - s) + __ldg(p + s)) - (__ldg(p - 2 * s) + __ldg(p + 2 * s)) - T(30) * c0) *
-         i12h2;
-}
-
-// D_b(D_a U): tensor product of two first-derivative stencils (16 points)
-template <typename T>
-__device__ __forceinline__ T dmix(const T* __restrict__ p, long long sa, long long sb, T i144) {
-  auto row = [&](long long o) {
-    const T* q = p + o;
-    return (__ldg(q - 2 * sa) - __ldg(q + 2 * sa)) + T(8) * (__ldg(q + sa) - __ldg(q - sa));
-  };
-  return ((row(-2 * sb) - row(2 * sb)) + T(8) * (row(sb) - row(-sb))) * i144;
-}
-
-// 6th difference along one direction: U-3 - 6U-2 + 15U-1 - 20U0 + 15U+1 - 6U+2 + U+3
-template <typename T>
-__device__ __forceinline__ T delta6(const T* __restrict__ p, long long s, T c0) {
-  return (__ldg(p - 3 * s) + __ldg(p + 3 * s)) - T(6) * (__ldg(p - 2 * s) + __ldg(p + 2 * s)) +
-         T(15) * (__ldg(p - s) + __ldg(p + s)) - T(20) * c0;
-}
-
-template <typename T>
-__device__ __forceinline__ T ko_all(const T* __restrict__ p, long long sy, long long sz, T c0,
-                                    const T* kc) {
-  return kc[0] * delta6(p, 1, c0) + kc[1] * delta6(p, sy, c0) + kc[2] * delta6(p, sz, c0);
-}
 
 // (by its exponent bits: a double comparison takes the FP64 pipe, 1% of an FP64
 // CCZ4 stage)
@@ -262,15 +225,14 @@ __device__ __forceinline__ void write_fields(const PatchArgs<T>& a, const StageA
 }
 
 // ------------------------------------------------------------ launch plumbing
-struct Launch {
-  dim3 grid, block;
-};
-
 // Programmatic stream serialization: the launch of a kernel that waits for its
 // predecessor itself overlaps the predecessor's end (its blocks are placed when
 // the last of the predecessor's has exited, before its memory is flushed).
 // Every kernel launched by launch_after() calls wait_predecessor() before it
-// reads or writes global memory; without an explicit trigger, so that no
+// reads or writes global memory, and reads what its predecessor may have
+// written by plain loads: its lifetime begins before those writes are flushed,
+// so to it they are not the read-only data that __ldg (which a compiler may
+// also move above the wait) is for.  Without an explicit trigger, so that no
 // waiting block takes a place from a running one (triggering at the start made
 // FP64 wave stages of 24^3 twice as slow).  Chains of small stages gain most:
 // 16^3 wave stage 6.2 -> 3.3 us.

@@ -158,7 +158,7 @@ __device__ __forceinline__ T flux_speed(const T* q, int d, const MhdCoef<T>& mc,
 // the six cells p-2..p+3, F+- = (F(U) +- S U)/2 at each cell, F+ reconstructed
 // from the left (cells p-2..p+2) plus F- from the right (cells p-1..p+3).
 template <typename T, int VAR>
-__device__ __forceinline__ void face_flux_split(const T* __restrict__ p, long long F, long long s,
+__device__ __forceinline__ void face_flux_split(const T* p, long long F, long long s,
                                                 int d, const MhdCoef<T>& mc, T* Fout) {
   const T eps = by_dir(d, mc.eps[0], mc.eps[1], mc.eps[2]);
   T Uc[6][8], Fc[6][8];
@@ -166,7 +166,7 @@ __device__ __forceinline__ void face_flux_split(const T* __restrict__ p, long lo
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
 #pragma unroll
-    for (int f = 0; f < 8; ++f) Uc[c][f] = __ldg(p + f * F + (c - 2) * s);
+    for (int f = 0; f < 8; ++f) Uc[c][f] = p[f * F + (c - 2) * s];
     const T sp = flux_speed(Uc[c], d, mc, Fc[c]);
     S = sp > S ? sp : S;
   }
@@ -424,7 +424,7 @@ __device__ __forceinline__ void mhd_march(const PatchArgs<T>& a, const StageArgs
             w[o] = sm.ring[sl[1]][f * NC + lc + (o - 2) * lst];
           } else {
             const T* q = plane + gc + (o - 2) * gst + 2 * f * a.sf;
-            w[o] = P(__ldg(q), __ldg(q + a.sf));
+            w[o] = P(*q, q[a.sf]);
           }
         }
         weno_edges<VAR, T, P>(w, eps, mc, er[f], el[f]);
@@ -471,7 +471,7 @@ __device__ __forceinline__ void mhd_march(const PatchArgs<T>& a, const StageArgs
             w[o] = sm.ring[row ? sl[o] : sl[1]][f * NC + lz_ + (row ? 0 : (o - 2) * CW)];
           } else {
             const T* q = plane + (row ? a.sz : 0) + gz + (o - 2) * (row ? a.sz : a.sy) + 2 * f * a.sf;
-            w[o] = P(__ldg(q), __ldg(q + a.sf));
+            w[o] = P(*q, q[a.sf]);
           }
         }
         weno_edges<VAR, T, P>(w, eps, mc, r[f], l[f]);
@@ -557,7 +557,7 @@ __device__ __forceinline__ void mhd_march(const PatchArgs<T>& a, const StageArgs
               const P v = sm.ring[sl[1]][(f / 2) * NC + lz_];
               cen[f] = f % 2 ? v.y : v.x;
             } else {
-              cen[f] = __ldg(a.us + f * a.sf + c);
+              cen[f] = a.us[f * a.sf + c];
             }
           }
           const Images im = ghost_images(a, s, i, j, k);
@@ -709,7 +709,7 @@ __global__ void __launch_bounds__(MX * SY, sizeof(T) == 4 && VAR == 2 ? 2 : 1)
         r -= (Fxp[f] - Fx[f]) * mc.idx[0];
         r -= (fy[ty + 1][tx][f] - Fy[f]) * mc.idx[1];
         r -= (Fz[f] - Fzm[f]) * mc.idx[2];
-        q[f] = write_field(a, s, im, f, c, i, j, k, __ldg(a.us + f * a.sf + c), r);
+        q[f] = write_field(a, s, im, f, c, i, j, k, a.us[f * a.sf + c], r);
         Fzm[f] = Fz[f];
       }
       if (a.rate) rate = fmax(rate, cell_rate(q, mc));

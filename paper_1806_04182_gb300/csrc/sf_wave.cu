@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(kMarchX * kMarchY, 3)
 #pragma unroll
   for (int f = 0; f < 5; ++f)
 #pragma unroll
-    for (int q = 1; q < 4; ++q) w[f][q] = __ldg(a.us + (c + f * sf + (q - 4) * sz));
+    for (int q = 1; q < 4; ++q) w[f][q] = a.us[c + f * sf + (q - 4) * sz];
   const float* lc = ring + (ty + 3) * CW + tx + 3;
   // planes k0 .. k0 + 2 have landed
   asm volatile("cp.async.wait_group 2;" ::: "memory");

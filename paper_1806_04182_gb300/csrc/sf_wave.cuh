@@ -67,14 +67,14 @@ __device__ __forceinline__ void wave_rhs(const PatchArgs<T>& a, Ld&& ld, const T
 
 // The same with every read from global memory (u: the point in field 0).
 template <typename T, bool ADJ>
-__device__ __forceinline__ void wave_point(const PatchArgs<T>& a, const T* __restrict__ u, T v[5],
+__device__ __forceinline__ void wave_point(const PatchArgs<T>& a, const T* u, T v[5],
                                            T r[5]) {
 #pragma unroll
-  for (int f = 0; f < 5; ++f) v[f] = __ldg(u + f * a.sf);
+  for (int f = 0; f < 5; ++f) v[f] = u[f * a.sf];
   wave_rhs<T, ADJ>(
       a,
       [&](int f, int d, int o) {
-        return __ldg(u + f * a.sf + o * (d == 0 ? 1LL : (d == 1 ? a.sy : a.sz)));
+        return u[f * a.sf + o * (d == 0 ? 1LL : (d == 1 ? a.sy : a.sz))];
       },
       v, r);
 }

@@ -66,13 +66,13 @@ struct Cross {
 // Stencil source reading the ghosted SoA arrays in global memory.
 template <typename T, int SY, int SZ>
 struct GlobalSrc {
-  const T* __restrict__ u;  // centre of field 0
+  const T* u;  // centre of field 0
   long long F, sy_, sz_;
   __device__ __forceinline__ long long sy() const { return SY ? (long long)SY : sy_; }
   __device__ __forceinline__ long long sz() const { return SZ ? (long long)SZ : sz_; }
   __device__ __forceinline__ const T* p(int f) const { return u + f * F; }
-  __device__ __forceinline__ T ld(const T* q) const { return __ldg(q); }
-  __device__ __forceinline__ T centre(int f) const { return __ldg(u + f * F); }
+  __device__ __forceinline__ T ld(const T* q) const { return *q; }
+  __device__ __forceinline__ T centre(int f) const { return u[f * F]; }
   __device__ __forceinline__ void begin(int) {}   // called before field f's first stencil
   __device__ __forceinline__ void finish() {}     // called once at the end
 };

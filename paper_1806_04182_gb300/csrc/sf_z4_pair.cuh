@@ -153,7 +153,7 @@ struct PairSrc {
   static constexpr int KS = C::KS;
   static constexpr int kY = C::XB;            // box row, floats
   static constexpr int kZ = C::XB * C::TY;    // box plane, floats
-  const float* __restrict__ u;  // global stage input at point i, field 0
+  const float* u;  // global stage input at point i, field 0
   long long F;
   const PairCoef* pc;
   float* tiles;

@@ -107,7 +107,7 @@ struct TmaSrc {
   static constexpr int kSlots = KS;
   static constexpr int kSlotFloats = C::kSlotFloats;
   static constexpr int kBoxBytes = C::kBoxBytes;
-  const float* __restrict__ u;  // global stage input at this point, field 0
+  const float* u;  // global stage input at this point, field 0
   long long F;
   float* tiles;
   uint64_t* full;
@@ -123,7 +123,7 @@ struct TmaSrc {
   __device__ __forceinline__ static constexpr long long sz() { return XB * TY; }
   __device__ __forceinline__ const float* p(int) const { return tiles + cur * kSlotFloats + local; }
   __device__ __forceinline__ float ld(const float* q) const { return *q; }
-  __device__ __forceinline__ float centre(int f) const { return __ldg(u + f * F); }
+  __device__ __forceinline__ float centre(int f) const { return u[f * F]; }
 
   // leader: load field use j into its slot once the previous occupant
   // (use j - kSlots) has been released by every warp
