@@ -8,11 +8,14 @@
 // 36% of them on patches of 16 to 64 points a side and 25% on 48^3 (96 mixed
 // patches 11.6 ms per RK4 step, eight 48^3 patches with halo exchange 1.59; with
 // the other two alone 10.0 and 1.36).  A launch takes rounds of one tile per
-// SM, and a round of the three shapes 23.9, 24.4 and 25.5 us a stage, so a patch
-// takes the shape of the least rounds x time.  Stage of 80 x 24 x 23 (138, 108
-// or 90 tiles: one round) 23.9, 24.0, 25.1 us; 48^3 (two rounds) 47.5, 48.4,
-// 51.7; 60 x 20 x 88 (3, 2, 2) 69, 50, 55; 70 x 50 x 61 (5, 5, 4) 113, 107, 96.
-// (By tiles x time instead the first two took the deep tiles.)
+// SM, a round of the three shapes 40 : 41 : 43, and a last round that does not
+// fill the SMs 0.7 to 0.95 of a full one, so a patch takes the shape of the
+// least rounds x time.  Stage of 80 x 24 x 23 (138, 108 or 90 tiles: one
+// round) 23.9, 24.0, 25.1 us; 48^3 (288, 288, 216) 47.5, 48.4, 51.7; 60 x 20 x 88
+// (352, 264, 264) 69, 50, 55; 33 x 21 x 68 (272, 204, 153) 43, 42, 41; 70 x 50 x
+// 61 (732, 651, 560) 113, 107, 96.  Over 60 sizes of 16 to 96 points a side the
+// rule's shape takes 0.4% longer than the best of the three (the least tiles
+// x time, 2.2%; 32 x 16 x 1 always, 8.6%) and none longer than 32 x 16 x 1.
 #include <algorithm>
 
 #include "sf_z4_pair.cuh"
@@ -25,17 +28,18 @@ static long long pair_tiles(const sf_patch& p, int w) {
   for (int d = 0; d < 3; ++d) n *= (p.n[d] + kPairShapes[w][d] - 1) / kPairShapes[w][d];
   return n;
 }
-static long long pair_rounds(long long tiles) {
-  const long long sms = std::max(1, sm_count());
-  return (tiles + sms - 1) / sms;
+static double pair_rounds(long long tiles) {
+  const long long sms = std::max(1, sm_count()), full = tiles / sms, rest = tiles % sms;
+  if (full == 0) return 1.0;
+  return (double)full + (rest ? 0.7 + 0.25 * (double)rest / (double)sms : 0.0);
 }
 
 int z4_pair_shape(const sf_patch& p) {
   int best = 0;
-  long long cost = -1;
+  double cost = 0.0;
   for (int w = 0; w < 3; ++w) {
-    const long long c = pair_rounds(pair_tiles(p, w)) * kPairTime[w];
-    if (cost < 0 || c < cost) {
+    const double c = pair_rounds(pair_tiles(p, w)) * kPairTime[w];
+    if (w == 0 || c < cost) {
       cost = c;
       best = w;
     }
@@ -53,7 +57,7 @@ void z4_pair_batch_shapes(const std::vector<const sf_patch*>& ps, std::vector<in
   for (int w = 0; w < 3; ++w) {
     long long n = 0;
     for (const sf_patch* p : ps) n += pair_tiles(*p, w);
-    const double c = (double)(pair_rounds(n) * kPairTime[w]);
+    const double c = pair_rounds(n) * kPairTime[w];
     if (w == 0 || c < cost) {
       cost = c;
       best = w;
@@ -67,7 +71,7 @@ void z4_pair_batch_shapes(const std::vector<const sf_patch*>& ps, std::vector<in
     n += mixed[q] == 2 ? t2 : t1;
     work += std::min(t2 * kPairTime[2], t1 * kPairTime[1]);
   }
-  if ((double)pair_rounds(n) * (double)work / (double)n < cost)
+  if (pair_rounds(n) * (double)work / (double)n < cost)
     shapes = mixed;
   else
     shapes.assign(ps.size(), best);
