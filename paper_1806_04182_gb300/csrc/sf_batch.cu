@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? 3 : 2) batch_stage_kerne
     for (int k = w.z0; k < zend; ++k) {
       const long long c = (long long)(k + g) * a.sz + (long long)(j + g) * a.sy + (i + g);
       if (system == SF_Z4) {
-        GlobalSrc<T, 0, 0> src{a.us + c, a.sf, a.sy, a.sz};
+        GlobalSrc<T, 0, 0, LOP> src{a.us + c, a.sf, a.sy, a.sz};
         const Images im = ghost_images(a, s, i, j, k);
         z4_cell<T, H, LOP>(a, zc, src, [&](int f, T r, T) { rbuf[f * 128 + threadIdx.x] = r; });
         write_fields<T, 25>(a, s, im, c, i, j, k, rbuf + threadIdx.x, 128);

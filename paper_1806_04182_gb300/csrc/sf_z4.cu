@@ -42,7 +42,7 @@ __global__ void __launch_bounds__(128, MINB)
   const long long sy = SY ? (long long)SY : a.sy;
   const long long sz = SZ ? (long long)SZ : a.sz;
   const long long c = (long long)(k + g) * sz + (long long)(j + g) * sy + (i + g);
-  GlobalSrc<T, SY, SZ> src{a.us + c, a.sf, a.sy, a.sz};
+  GlobalSrc<T, SY, SZ, LOP> src{a.us + c, a.sf, a.sy, a.sz};
   const Images im = ghost_images(a, s, i, j, k);
   const int tid = threadIdx.y * 32 + threadIdx.x;
   z4_cell<T, H, LOP>(a, zc, src, [&](int f, T r, T) { rbuf[f * 128 + tid] = r; });

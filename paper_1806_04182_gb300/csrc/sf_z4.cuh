@@ -63,16 +63,28 @@ struct Cross {
   T adv;    // beta^k d_k U: centred D_k, or one-sided by the sign of beta^k
 };
 
-// Stencil source reading the ghosted SoA arrays in global memory.
-template <typename T, int SY, int SZ>
+// Stencil source reading the ghosted SoA arrays in global memory.  LOP: the
+// one-sided form, whose float instances read in program order (asm volatile):
+// left to the compiler's order they spill more (412 instead of 272 bytes with
+// FP64 islands; 30 x 25 x 90 step 350 against 334 us, 61 x 47 x 53 with
+// double-word islands 413 against 413).  The centred form is no faster so.
+template <typename T, int SY, int SZ, bool LOP>
 struct GlobalSrc {
   const T* u;  // centre of field 0
   long long F, sy_, sz_;
   __device__ __forceinline__ long long sy() const { return SY ? (long long)SY : sy_; }
   __device__ __forceinline__ long long sz() const { return SZ ? (long long)SZ : sz_; }
   __device__ __forceinline__ const T* p(int f) const { return u + f * F; }
-  __device__ __forceinline__ T ld(const T* q) const { return *q; }
-  __device__ __forceinline__ T centre(int f) const { return u[f * F]; }
+  __device__ __forceinline__ T ld(const T* q) const {
+    if constexpr (LOP && sizeof(T) == 4) {
+      T v;
+      asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(q));
+      return v;
+    } else {
+      return *q;
+    }
+  }
+  __device__ __forceinline__ T centre(int f) const { return ld(u + f * F); }
   __device__ __forceinline__ void begin(int) {}   // called before field f's first stencil
   __device__ __forceinline__ void finish() {}     // called once at the end
 };
