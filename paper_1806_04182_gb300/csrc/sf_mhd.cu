@@ -294,14 +294,15 @@ __device__ __forceinline__ void ssp_write(const PatchArgs<T>& a, const StageArgs
 // each where 8 get 255 (float, 9 warps: 1410 us per 128^3 step, 8: 1155).
 // 128^3 SSP-RK3 step with CFL rate, against a kernel that reconstructed each
 // cell once per face and side in tiles of 31 x 11 (float) and 31 x 7 outputs:
-// double 54.4 -> 20.3 ms, float 2.22 -> 0.91 ms.
+// double 54.4 -> 20.8 ms, float 2.23 -> 0.92 ms.
 //
 // A block's work is one chunk of mz planes of one column of tiles or, in
 // double where that is less, an even share of all columns laid end to end,
 // whose boundaries fall between planes: a launch of as many blocks as the GPU
 // holds, all ending together (128^3: 36 columns of 128 planes over 152 SMs,
-// 20.9 -> 20.3 ms).  float keeps to chunks: the loop over the columns of a
-// share costs registers that its planes need (915 -> 965 us).
+// 20.9 -> 20.3 ms when a field took 41 operations).  float keeps to chunks:
+// the loop over the columns of a share costs registers that its planes need
+// (915 -> 965 us).
 constexpr int MX = 32;
 struct MhdWork {
   int mz;      // planes of a chunk; 0: even shares

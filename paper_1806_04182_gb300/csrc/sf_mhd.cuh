@@ -97,14 +97,22 @@ __device__ __forceinline__ double nrecip1(double x) {
 }
 __device__ __forceinline__ R2 nrecip2(R2 x) { return R2(nrecip1<false>(x.x), nrecip1<false>(x.y)); }
 
-// Square root of a non-negative value; float: h = x rsqrt(x) and one Newton
-// step h (3/2 - h rsqrt(x) / 2).
-__device__ __forceinline__ F2 sqrt2(F2 x) {
+// Square root, 0 of a negative value (of a rounding error: the discriminant's,
+// or that of the sum under the root of the signal speed of a state with
+// negative pressure); NaN stays.  float: h = x rsqrt(x) and one Newton step h
+// (3/2 - h rsqrt(x) / 2), x no less than 1e-37.
+__device__ __forceinline__ F2 root2(F2 x) {
+  auto up = [](float v) {
+    float r;
+    asm("max.NaN.f32 %0, %1, 0f02081CEA;" : "=f"(r) : "f"(v));  // 1e-37
+    return r;
+  };
   auto rs = [](float v) {
     float y;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(fmaxf(v, 1e-37f)));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(v));
     return y;
   };
+  x = F2(up(x.x), up(x.y));
   const F2 y(rs(x.x), rs(x.y));
   const F2 h = mul2(x, y);
   return fma2(h, fma2(mul2(y, F2(-0.5f)), h, F2(0.5f)), h);
@@ -120,26 +128,11 @@ __device__ __forceinline__ double sqrt1(double x) {
   const double h = __dmul_rn(x, y), e = __fma_rn(-h, y, 1.0);
   return __fma_rn(__dmul_rn(h, e), __fma_rn(0.375, e, 0.5), h);
 }
-__device__ __forceinline__ R2 sqrt2(R2 x) { return R2(sqrt1(x.x), sqrt1(x.y)); }
-
-// max(x, 0) per lane, NaN kept out of the comparison; double: by the sign
-// bit, off the FP64 pipe.
-__device__ __forceinline__ F2 pos2(F2 x) { return F2(fmaxf(x.x, 0.0f), fmaxf(x.y, 0.0f)); }
-__device__ __forceinline__ R2 pos2(R2 x) {
-  return R2(__double2hiint(x.x) < 0 ? 0.0 : x.x, __double2hiint(x.y) < 0 ? 0.0 : x.y);
-}
-// the same, but NaN stays (the sum under the root of the signal speed: of a
-// state with negative pressure it is a rounding error of either sign)
-__device__ __forceinline__ float nonneg(float x) {
-  float r;
-  asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ double nonneg(double x) {
+__device__ __forceinline__ double nonneg(double x) {  // by the sign bit, off the FP64 pipe
   return (unsigned)__double2hiint(x) - 0x80000000u < 0x7ff00000u ? 0.0 : x;  // finite, < 0
 }
-__device__ __forceinline__ F2 nonneg2(F2 x) { return F2(nonneg(x.x), nonneg(x.y)); }
-__device__ __forceinline__ R2 nonneg2(R2 x) { return R2(nonneg(x.x), nonneg(x.y)); }
+__device__ __forceinline__ R2 root2(R2 x) { return R2(sqrt1(nonneg(x.x)), sqrt1(nonneg(x.y))); }
+
 __device__ __forceinline__ F2 abs2(F2 x) { return F2(fabsf(x.x), fabsf(x.y)); }
 __device__ __forceinline__ R2 abs2(R2 x) { return R2(fabs(x.x), fabs(x.y)); }
 // the larger of two non-negative values; double: as integers (their bits are
@@ -150,6 +143,11 @@ __device__ __forceinline__ double larger(double a, double b) {
 }
 
 // ------------------------------------------------------------ reconstruction
+// 2^-floor(log2 m) of a normal m < 2^127
+__device__ __forceinline__ float inv_pow2(float m) {
+  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
+}
+
 // Nonlinear weights P_k (without their linear weights) from E_k = eps + beta_k,
 // up to a common factor.
 //
@@ -158,12 +156,10 @@ __device__ __forceinline__ double larger(double a, double b) {
 // power of two of the largest first, so that the largest P_k lies in [1, 4)
 // whatever the units.  Where a product leaves the range of that scale (E_k
 // above 9e18: jumps of 3e9) P_k = (E_min / E_k)^2, in [0, 1], the largest 1; a
-// weight below the range of a float is nil, as 1/E_k^2 is.  (That form for all
-// cells: 1.3% more on the 128^3 step.)
-// 2^-floor(log2 m) of a normal m < 2^127
-__device__ __forceinline__ float inv_pow2(float m) {
-  return __int_as_float(0x7f000000 - (__float_as_int(m) & 0x7f800000));
-}
+// weight below the range of a float is nil, as 1/E_k^2 is.  (128^3 step 919 us;
+// without that form 911, with it for all cells 931, the test shared by two or
+// four pairs of fields, whose values then wait for it in registers, 960 and
+// 1056.)
 template <int VAR>
 __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
                                              F2& p1, F2& p2) {
@@ -333,7 +329,7 @@ __device__ __forceinline__ void llf_flux2(const P* q, T gamma, T* F) {
   const P na2 = mul2(mul2(P(gamma), pr), nir);
   const P h = mul2(P(T(-0.5)), fma2(B2, nir, na2));
   const P disc = fma2(neg2(na2), mul2(bd2, nir), mul2(h, h));
-  const P cf = sqrt2(nonneg2(add2(sqrt2(pos2(disc)), h)));
+  const P cf = root2(add2(root2(disc), h));
   const T S = larger(fabs(nv[D].x) + cf.x, fabs(nv[D].y) + cf.y);
   auto out = [&](int f, P nf) { F[f] = fma(-S, q[f].y - q[f].x, -nf.x - nf.y); };
   F[0] = fma(-S, q[0].y - q[0].x, Sd.x + Sd.y);
