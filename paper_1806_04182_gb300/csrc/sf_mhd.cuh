@@ -164,20 +164,34 @@ template <int VAR>
 __device__ __forceinline__ void weno_weights(F2 e0, F2 e1, F2 e2, const MhdCoef<float>& mc, F2& p0,
                                              F2& p1, F2& p2) {
   if constexpr (VAR == 1) {
-    // 1 + (tau / E_k)^q, times the q-th power of a scale: beyond ratios of 2^30
-    // (a jump of 2 beside a uniform state on 128 cells) the inverse power of
-    // two of the largest, so that the weights and their sums stay in range
+    // 1 + (tau / E_k)^q, times the q-th power of a scale u: beyond ratios of
+    // 2^30 (a jump of 2 beside a uniform state on 128 cells) the inverse power
+    // of two of the largest, so that the weights and their sums stay in range.
+    // q = 2 in a branch of its own for all of it (64^3 step 354 -> 247 us; 318
+    // without the scale and with the power chosen value by value)
     const F2 tau = abs2(sub2(e0, e2));
-    auto lane = [&](float t, float a, float b, float c, float& pa, float& pb, float& pc) {
-      auto ratio = [&](float e) { return fminf(t / e, 1.5e38f); };
-      const float ra = ratio(a), rb = ratio(b), rc = ratio(c), m = fmaxf(fmaxf(ra, rb), rc);
-      const float u = m < 0x1p30f ? 1.0f : inv_pow2(m), one = wz_pow(u, mc.q);
-      pa = one + wz_pow(ra * u, mc.q);
-      pb = one + wz_pow(rb * u, mc.q);
-      pc = one + wz_pow(rc * u, mc.q);
+    auto ratio = [&](F2 e) { return F2(fminf(tau.x / e.x, 1.5e38f), fminf(tau.y / e.y, 1.5e38f)); };
+    F2 r0 = ratio(e0), r1 = ratio(e1), r2 = ratio(e2);
+    auto scale = [](float a, float b, float c) {
+      const float m = fmaxf(fmaxf(a, b), c);
+      return m < 0x1p30f ? 1.0f : inv_pow2(m);
     };
-    lane(tau.x, e0.x, e1.x, e2.x, p0.x, p1.x, p2.x);
-    lane(tau.y, e0.y, e1.y, e2.y, p0.y, p1.y, p2.y);
+    const F2 u(scale(r0.x, r1.x, r2.x), scale(r0.y, r1.y, r2.y));
+    r0 = mul2(r0, u);
+    r1 = mul2(r1, u);
+    r2 = mul2(r2, u);
+    if (mc.q == 2.0f) {
+      const F2 one = mul2(u, u);
+      p0 = fma2(r0, r0, one);
+      p1 = fma2(r1, r1, one);
+      p2 = fma2(r2, r2, one);
+    } else {
+      auto power = [&](F2 r) { return F2(wz_pow(r.x, mc.q), wz_pow(r.y, mc.q)); };
+      const F2 one = power(u);
+      p0 = add2(one, power(r0));
+      p1 = add2(one, power(r1));
+      p2 = add2(one, power(r2));
+    }
   } else {
     p0 = mul2(e1, e2);
     p1 = mul2(e0, e2);
