@@ -1,7 +1,7 @@
 // The two-point CCZ4 tile (sf_z4_pair.cuh) over the tiles of many patches of any
-// size, in one launch.  A level of equal patches takes one shape (kPairShapes)
-// and that shape's kernel; patches that differ take the wide or the deep one
-// each, in a kernel that holds both tile bodies.  (A kernel with all three
+// size, in one launch: all in one shape (kPairShapes) and that shape's kernel,
+// or, where that saves rounds, each in the wide or the deep one, in a kernel
+// that holds both tile bodies (z4_pair_batch_shapes).  (A kernel with all three
 // spills: 96 mixed patches 9.96 instead of 9.52 ms, eight 48^3 patches 1.41
 // instead of 1.36.)
 #include <algorithm>
