@@ -136,7 +136,7 @@ __device__ __forceinline__ R2 root2(R2 x) { return R2(sqrt1(nonneg(x.x)), sqrt1(
 __device__ __forceinline__ F2 abs2(F2 x) { return F2(fabsf(x.x), fabsf(x.y)); }
 __device__ __forceinline__ R2 abs2(R2 x) { return R2(fabs(x.x), fabs(x.y)); }
 // the larger of two non-negative values; double: as integers (their bits are
-// ordered alike, NaN above all)
+// ordered alike)
 __device__ __forceinline__ float larger(float a, float b) { return a > b ? a : b; }
 __device__ __forceinline__ double larger(double a, double b) {
   return __longlong_as_double(max(__double_as_longlong(a), __double_as_longlong(b)));
